@@ -1,0 +1,308 @@
+// k_query_set.cu -- the set stage (Algorithm 2's union per table and
+// intersection across tables) of the queries whose masks leave many candidate
+// sets, 32 * QW of them at a time.
+//
+// The query kernel hands such a query over as its R per-table cell masks.  A
+// block takes 32 * QW queries and transposes their masks in shared memory, so
+// that T[r][cell] holds one bit per query: bit q = cell is hit in table r for
+// query q.  A set i then needs one shared-memory read per table for all of
+// them,
+//     acc = registered(i) AND T[0][phi_0(i)] AND ... AND T[R-1][phi_{R-1}(i)],
+// instead of one bit test per table and query.  A warp takes 256 consecutive
+// IDs (32 lanes x 8), transposes each 32-ID x 32-query block of acc back with
+// five shuffles, and every lane stores 8 words (one 32-byte sector) of its
+// query's K-bit bitmap, which the gather expands.
+//
+// What bounds it: the shared-memory pipe.  32 IDs x 128 queries cost R 16-byte
+// reads a lane at random cells (8.6 wavefronts each, measured) and 20 shuffles;
+// ncu shows 64% of the pipe's wavefronts and 3 blocks an SM.  Measured, set
+// stage with the probes before it, against one query per warp in the query
+// kernel: 1e5 conjunctive queries over 1e5 documents (R = 8, B = 320) 11.7 ms
+// -> 0.26 (probes) + 0.89; 1e4 over 5e5 documents (R = 6, B = 1000; no
+// per-warp bitmap there, so the start scanned all IDs twice) 85.4 ms -> 0.03 +
+// 0.54; 16 queries over 1e5 documents 202 us -> 28.
+//
+// Groups of 128 queries are the widest whose T leaves two blocks an SM room;
+// with fewer than 65 or 33 queries narrower groups read less of T per ID.
+#include "rambo_impl.cuh"
+
+namespace rgb {
+
+constexpr int QS_THREADS = 256;
+constexpr int QS_WARPS = QS_THREADS / 32;
+constexpr uint32_t QS_IDS = 256;                  // IDs a warp takes at a time
+constexpr size_t QS_SMEM_TWO = 100 * 1024;        // two blocks an SM
+constexpr size_t QS_SMEM_MOST = 200 * 1024;
+
+struct SetShared {
+    uint32_t* dst[128];      // bitmaps of the group's queries
+    uint32_t q[128];         // their indexes
+    uint32_t cnt[128];       // their set bits in this item
+    uint64_t warp[QS_WARPS];
+    bool last;
+};
+
+// 32x32 bit transpose across the warp: lane l's bit b becomes lane b's bit l.
+// Step S swaps the S-bit halves of lane pairs S apart; a lane keeps the bits
+// under its mask and takes the others from its partner's word, rotated.
+struct Transpose {
+    uint32_t keep[5];
+    uint32_t rot[5];
+    __device__ __forceinline__ explicit Transpose(unsigned lane) {
+        const uint32_t low[5] = {0x0000ffffu, 0x00ff00ffu, 0x0f0f0f0fu, 0x33333333u, 0x55555555u};
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+            const unsigned S = 16u >> i;
+            keep[i] = (lane & S) ? ~low[i] : low[i];
+            rot[i] = (lane & S) ? 32 - S : S;
+        }
+    }
+    template <int I>
+    __device__ __forceinline__ uint32_t step(uint32_t x) const {
+        const uint32_t y = __shfl_xor_sync(FULL, x, 16 >> I);
+        return (x & keep[I]) | (__funnelshift_l(y, y, rot[I]) & ~keep[I]);
+    }
+    __device__ __forceinline__ uint32_t operator()(uint32_t x) const {
+        return step<4>(step<3>(step<2>(step<1>(step<0>(x)))));
+    }
+};
+
+template <int QW>
+__device__ __forceinline__ void load_t(const uint32_t* t, uint32_t (&v)[QW]) {
+    if constexpr (QW == 1) {
+        v[0] = *t;
+    } else if constexpr (QW == 2) {
+        const uint2 x = *reinterpret_cast<const uint2*>(t);
+        v[0] = x.x, v[1] = x.y;
+    } else {
+        const uint4 x = *reinterpret_cast<const uint4*>(t);
+        v[0] = x.x, v[1] = x.y, v[2] = x.z, v[3] = x.w;
+    }
+}
+
+// Queries [g * 32 * QW, ...) of the deferred list against IDs [256 * c0, 256 * c1).
+template <int QW>
+__device__ __forceinline__ void set_item(const IndexView& ix, const QueryOut& o, uint64_t nd, uint64_t g, uint32_t c0,
+                                         uint32_t c1, uint32_t* T, SetShared& sh) {
+    const unsigned lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t W = ix.W, RS = ix.R * ix.S;
+    const Transpose transpose(lane);
+    const uint64_t slot0 = g * 32 * QW + lane;
+    if (threadIdx.x < 32 * QW) {
+        // where the queries' bitmaps go (null: no query)
+        const uint64_t slot = g * 32 * QW + threadIdx.x;
+        sh.dst[threadIdx.x] = slot < nd ? o.stage + slot * set_pitch(ix.K) : nullptr;
+        sh.q[threadIdx.x] = slot < nd ? o.dq[slot] : 0u;
+        sh.cnt[threadIdx.x] = 0;
+    }
+    // masks to T, up to four words of a table at a time (rows of S words, S = 1, 2 or a multiple of 4)
+    const uint32_t vec = ix.S < 4 ? ix.S : 4, quads = ix.S / vec;
+    for (uint32_t p = wid; p < ix.R * quads; p += QS_WARPS) {
+        const uint32_t r = p / quads, w0 = (p - r * quads) * vec;
+        uint32_t x[QW][4];
+#pragma unroll
+        for (int j = 0; j < QW; ++j) {
+            const uint32_t* m = o.dmask + (slot0 + 32 * j) * RS + r * ix.S + w0;
+            uint4 q = make_uint4(0, 0, 0, 0);
+            if (slot0 + 32 * j < nd) {
+                if (vec == 4) q = __ldg(reinterpret_cast<const uint4*>(m));
+                else q.x = __ldg(m), q.y = vec == 2 ? __ldg(m + 1) : 0u;
+            }
+            x[j][0] = q.x, x[j][1] = q.y, x[j][2] = q.z, x[j][3] = q.w;
+        }
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            if (w0 + v >= W || v >= (int)vec) break;
+            uint32_t* t = T + ((r * W + w0 + v) * 32 + lane) * QW;
+#pragma unroll
+            for (int j = 0; j < QW; ++j) x[j][v] = transpose(x[j][v]);
+            if constexpr (QW == 1) *t = x[0][v];
+            else if constexpr (QW == 2) *reinterpret_cast<uint2*>(t) = make_uint2(x[0][v], x[1][v]);
+            else *reinterpret_cast<uint4*>(t) = make_uint4(x[0][v], x[1][v], x[2][v], x[3][v]);
+        }
+    }
+    __syncthreads();
+    uint32_t tot[QW];
+#pragma unroll
+    for (int j = 0; j < QW; ++j) tot[j] = 0;
+    const uint4* phi = reinterpret_cast<const uint4*>(ix.phi);
+    for (uint32_t c = c0 + wid; c < c1; c += QS_WARPS) {
+        uint32_t out[QW][8];
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const uint64_t i0 = (uint64_t)c * QS_IDS + 128 * half + lane;
+            uint4 ph[4];
+            uint32_t reg[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const uint64_t i = i0 + 32 * u;
+                const bool in = i < ix.K;
+                ph[u] = in ? __ldg(phi + i) : make_uint4(0, 0, 0, 0);
+                reg[u] = in ? __ldg(ix.reg + (i >> 5)) : 0u;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const uint32_t cell[8] = {ph[u].x & 0xffffu, ph[u].x >> 16, ph[u].y & 0xffffu, ph[u].y >> 16,
+                                          ph[u].z & 0xffffu, ph[u].z >> 16, ph[u].w & 0xffffu, ph[u].w >> 16};
+                uint32_t acc[QW];
+#pragma unroll
+                for (int j = 0; j < QW; ++j) acc[j] = (reg[u] >> lane) & 1u ? ~0u : 0u;
+#pragma unroll
+                for (int r = 0; r < RF; ++r) {
+                    if (r < (int)ix.R) {
+                        uint32_t v[QW];
+                        load_t<QW>(T + (r * W * 32 + cell[r]) * QW, v);
+#pragma unroll
+                        for (int j = 0; j < QW; ++j) acc[j] &= v[j];
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < QW; ++j) out[j][4 * half + u] = transpose(acc[j]);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < QW; ++j) {
+            uint32_t* dst = sh.dst[32 * j + lane];
+            if (!dst) continue;
+            uint4* d = reinterpret_cast<uint4*>(dst + (uint64_t)c * 8);
+            d[0] = make_uint4(out[j][0], out[j][1], out[j][2], out[j][3]);
+            d[1] = make_uint4(out[j][4], out[j][5], out[j][6], out[j][7]);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) tot[j] += __popc(out[j][u]);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < QW; ++j)
+        if (tot[j]) atomicAdd(&sh.cnt[32 * j + lane], tot[j]);
+    __syncthreads();
+    if (threadIdx.x < 32 * QW && sh.cnt[threadIdx.x])
+        atomicAdd(o.qcount + sh.q[threadIdx.x], sh.cnt[threadIdx.x]);
+    __syncthreads();  // T and the counters are rewritten by the next item
+}
+
+template <int QW>
+__device__ __forceinline__ void set_items(const IndexView& ix, const QueryOut& o, uint64_t nd, uint32_t* T,
+                                          SetShared& sh) {
+    // items = query groups x ID ranges.  A range is a whole number of the
+    // block's steps (8 warps x 256 IDs); with few groups the ranges are
+    // short, so that four items per block keep the grid even
+    const uint32_t chunks = (uint32_t)((ix.K + QS_IDS - 1) / QS_IDS);
+    const uint32_t steps = (chunks + QS_WARPS - 1) / QS_WARPS;
+    const uint64_t groups = (nd + 32 * QW - 1) / (32 * QW);
+    const uint64_t want = (4ull * gridDim.x + groups - 1) / groups;
+    const uint32_t per = want < steps ? (steps + (uint32_t)want - 1) / (uint32_t)want : 1;
+    const uint32_t ranges = (steps + per - 1) / per;
+    for (uint64_t it = blockIdx.x; it < groups * ranges; it += gridDim.x) {
+        const uint64_t g = it / ranges;
+        const uint32_t r = (uint32_t)(it - g * ranges);
+        const uint32_t c0 = min(chunks, r * per * QS_WARPS), c1 = min(chunks, (r + 1) * per * QS_WARPS);
+        if (c0 < c1) set_item<QW>(ix, o, nd, g, c0, c1, T, sh);
+    }
+}
+
+// Exclusive scan of n counts by one block (16 a thread and round), out[n] the
+// total; the counts are read past L1 (other blocks added to them).
+__device__ __forceinline__ void scan_counts_block(const uint32_t* counts, uint64_t n, uint64_t* out, uint64_t carry,
+                                                  unsigned long long* total_out, uint64_t* s_warp) {
+    constexpr int PER = 16;
+    const unsigned lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (uint64_t base = 0; base < n; base += (uint64_t)QS_THREADS * PER) {
+        const uint64_t i0 = base + (uint64_t)threadIdx.x * PER;
+        uint32_t v[PER];
+        uint64_t sum = 0;
+#pragma unroll
+        for (int t = 0; t < PER; ++t) {
+            v[t] = i0 + t < n ? __ldcg(counts + i0 + t) : 0u;
+            sum += v[t];
+        }
+        uint64_t incl = sum;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint64_t y = __shfl_up_sync(FULL, incl, off);
+            if (lane >= (unsigned)off) incl += y;
+        }
+        if (lane == 31) s_warp[wid] = incl;
+        __syncthreads();
+        uint64_t pre = carry + incl - sum;
+#pragma unroll
+        for (int w = 0; w < QS_WARPS; ++w) {
+            const uint64_t x = s_warp[w];
+            if (w < (int)wid) pre += x;
+            carry += x;
+        }
+#pragma unroll
+        for (int t = 0; t < PER; ++t) {
+            if (i0 + t < n) out[i0 + t] = pre;
+            pre += v[t];
+        }
+        __syncthreads();  // the warp totals are rewritten by the next round
+    }
+    if (threadIdx.x == 0) {
+        out[n] = carry;
+        if (total_out) *total_out = carry;
+    }
+}
+
+__global__ void __launch_bounds__(QS_THREADS, 3)
+    k_set(IndexView ix, BatchView b, QueryOut o, int qw, int scan, uint64_t* __restrict__ id_offsets,
+          const uint64_t* __restrict__ base_dev, unsigned long long* __restrict__ total_out, DevStatus* st) {
+    extern __shared__ __align__(16) uint32_t qs_smem[];
+    __shared__ SetShared sh;
+    bv_resolve(b);
+    const uint64_t nd = st->n_handed;
+    if (st->err != NO_ERR) return;
+    if (nd) {
+        // narrower groups when the batch does not fill a wide one
+        if (qw >= 4 && nd > 64) set_items<4>(ix, o, nd, qs_smem, sh);
+        else if (qw >= 2 && nd > 32) set_items<2>(ix, o, nd, qs_smem, sh);
+        else set_items<1>(ix, o, nd, qs_smem, sh);
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        st->cursor = nd * set_pitch(ix.K);  // words staged: by this launch, and (spare) by the whole batch
+        st->spare[0] += nd * set_pitch(ix.K);
+        st->stage_count[1] += nd;
+    }
+    if (!scan) return;
+    // the block that finishes last lays out the answers
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) sh.last = atomicAdd(&st->set_done, 1ull) == gridDim.x - 1;
+    __syncthreads();
+    if (!sh.last) return;
+    __threadfence();
+    scan_counts_block(o.qcount, b.n, id_offsets, base_dev ? *base_dev : 0, total_out, sh.warp);
+}
+
+SetLaunch set_launch_shape(const IndexView& ix, int num_sms) {
+    SetLaunch sl{};
+    if (query_is_wide(ix.R, ix.S)) return sl;
+    const size_t one = (size_t)ix.R * ix.W * 32 * 4;  // a bit per cell for each of 32 queries
+    sl.qw = 4 * one <= QS_SMEM_TWO ? 4 : 2 * one <= QS_SMEM_TWO ? 2 : 4 * one <= QS_SMEM_MOST ? 4 : one <= QS_SMEM_MOST ? 1 : 0;
+    if (!sl.qw) return sl;
+    sl.smem = one * sl.qw;
+    const void* f = reinterpret_cast<const void*>(&k_set);
+    int per_sm = 0;
+    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)QS_SMEM_MOST) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, QS_THREADS, sl.smem) != cudaSuccess || per_sm < 1) {
+        cudaGetLastError();
+        sl.qw = 0;
+        return sl;
+    }
+    sl.blocks = per_sm * num_sms;
+    return sl;
+}
+
+cudaError_t launch_set(const SetLaunch& sl, const IndexView& ix, const BatchView& b, const QueryOut& o, int scan,
+                       uint64_t* id_offsets, const uint64_t* base_dev, unsigned long long* total_out, DevStatus* st,
+                       cudaStream_t s) {
+    if (b.n == 0 && !b.desc) return cudaSuccess;
+    // no more blocks than there can be items (b.n is the capacity of a descriptor batch)
+    const uint64_t steps = (ix.K + QS_IDS * QS_WARPS - 1) / (QS_IDS * QS_WARPS);
+    const uint64_t most = b.n * steps;
+    uint64_t blocks = (uint64_t)sl.blocks;
+    if (blocks > most) blocks = most < 1 ? 1 : most;
+    k_set<<<(unsigned)blocks, QS_THREADS, sl.smem, s>>>(ix, b, o, sl.qw, scan, id_offsets, base_dev, total_out, st);
+    return cudaGetLastError();
+}
+
+}  // namespace rgb

@@ -19,12 +19,16 @@ __global__ void k_status_reset(DevStatus* st) {
     st->err = NO_ERR;
     st->bad_pos = NO_ERR;
     st->ticket = 0;
+    st->gather_ticket = 0;
+    st->n_handed = 0;
+    st->set_done = 0;
+    st->n_long = 0;
+    st->ticket_long = 0;
     st->cursor = 0;
     st->keys_probed = 0;
     st->rows_read = 0;
     st->spare[0] = st->spare[1] = 0;
     st->stage_count[0] = st->stage_count[1] = st->stage_count[2] = st->stage_count[3] = 0;
-    st->gather_ticket = 0;
 }
 
 cudaError_t launch_status_reset(DevStatus* st, cudaStream_t s) {

@@ -128,7 +128,7 @@ struct rambo {
     // scratch
     DBuf<uint8_t> in_data;
     DBuf<uint64_t> in_off, in_ids, packed, qstart, scan_tmp, id_off;
-    DBuf<uint32_t> stage, qcount, ids, fill, perm, chist, nmask;
+    DBuf<uint32_t> stage, qcount, ids, fill, perm, chist, nmask, dmask, dq;
     DBuf<uint64_t> ckeys, coff;
     DBuf<uint32_t> brec;               // bucketed build: update records
     DBuf<unsigned long long> bfill;    // bucketed build: per-window fill counters + overflow flag
@@ -147,8 +147,14 @@ struct rambo {
     uint64_t launches = 0;
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};  // call start, query start/end, call end
     uint64_t last_err_item = 0;
-    // automatic block size: last (V, G, use_bitmap) resolved and its choice
-    int auto_key = -1, auto_wpb = 0, auto_per_sm = 0;
+    // block sizes and residency resolved for the query configuration tuned_cfg
+    struct Tuned {
+        int wpb = 0, per_sm = 0, per_sm_g = 0;                    // query kernel
+        int probe_wpb = 0, probe_per_sm = 0, probe_per_sm_g = 0, probe_per_sm_l = 0;  // probe kernel
+        SetLaunch set{};
+    } tuned;
+    rambo_query_config_t tuned_cfg{};
+    bool tuned_known = false;
     std::vector<rambo_plan_t*> plans;   // live plans (own or a server's) holding captured pointers
     unsigned char* na_base = nullptr;   // device address of the no-alloc query's fixed scratch
 
@@ -211,6 +217,8 @@ void free_handle(rambo* h) {
     h->perm.release();
     h->chist.release();
     h->nmask.release();
+    h->dmask.release();
+    h->dq.release();
     h->ckeys.release();
     h->brec.release();
     h->bfill.release();
@@ -287,7 +295,7 @@ void default_config(rambo* h) {
     h->cfg.words_per_lane = (uint32_t)V;
     h->cfg.lanes_per_key = (uint32_t)G;
     h->cfg.warps_per_block = 0;  // chosen per call from the occupancy
-    h->auto_key = -1;
+    h->tuned_known = false;
     h->cfg.blocks_per_sm = 0;
     h->cfg.set_stage = 0;
     h->cfg.visit_order = 2;
@@ -519,6 +527,81 @@ struct QueryDest {
     const uint64_t** out_off;
 };
 
+// The largest block that keeps at least 85% of the most warps any block size
+// can keep resident per SM (per_sm_of: blocks resident at w warps each).
+template <class F>
+bool pick_block(F per_sm_of, int& wpb, int& per_sm) {
+    int nb_of[4] = {0, 0, 0, 0}, best = 0;
+    for (int i = 0; i < 4; ++i) {
+        nb_of[i] = per_sm_of(8 >> i);
+        if (nb_of[i] * (8 >> i) > best) best = nb_of[i] * (8 >> i);
+    }
+    for (int i = 0; i < 4; ++i)
+        if (nb_of[i] > 0 && 100 * nb_of[i] * (8 >> i) >= 85 * best) {
+            wpb = 8 >> i;
+            per_sm = nb_of[i];
+            return true;
+        }
+    return false;
+}
+
+// Block sizes and blocks per SM of the kernels for the handle's configuration,
+// kept until the configuration changes (the occupancy queries behind them
+// cost more than a small batch's kernels).
+int resolve_residency(rambo* h, int use_bitmap) {
+    const int V = (int)h->cfg.words_per_lane, G = (int)h->cfg.lanes_per_key;
+    rambo::Tuned u{};
+    const int most = h->cfg.blocks_per_sm ? (int)h->cfg.blocks_per_sm : 1 << 20;
+    // the query kernel: the per-warp bitmap grows with K, so for large ID
+    // spaces shared memory, not registers, limits the residency and smaller
+    // blocks pack the SM more fully
+    const size_t spw = (size_t)query_smem_words_per_warp(h->R, h->S, h->K, use_bitmap) * 4;
+    auto query_at = [&](int w) { return query_max_blocks_per_sm(V, G, h->eta, false, w, spw * (size_t)w); };
+    if (h->cfg.warps_per_block) {
+        u.wpb = (int)h->cfg.warps_per_block;
+        u.per_sm = query_at(u.wpb);
+        if (u.per_sm < 1) return RAMBO_EINVAL;
+    } else if (!pick_block(query_at, u.wpb, u.per_sm)) {
+        return RAMBO_EINVAL;
+    }
+    if (u.per_sm > most) u.per_sm = most;
+    const int group = (int)h->cfg.warps_per_query;
+    if (use_bitmap && group != 1 && u.wpb > 1)
+        u.per_sm_g = std::min(most, query_max_blocks_per_sm(V, G, h->eta, true, u.wpb,
+                                                            query_group_smem_bytes(h->R, h->S, h->K, u.wpb, group)));
+    // the probe and set kernels serve the automatic set stage and staging form
+    // and the default row reads; other choices name what the query kernel does
+    if (h->cfg.set_stage == 0 && h->cfg.answer_staging == 0 && h->cfg.row_load == 7) u.set = set_launch_shape(h->view(), h->num_sms);
+    if (u.set.qw) {
+        auto probe_at = [&](int w) { return probe_max_blocks_per_sm(V, G, h->eta, PB_WARP, w, 0); };
+        bool ok = true;
+        if (h->cfg.warps_per_block) {
+            u.probe_wpb = (int)h->cfg.warps_per_block;
+            u.probe_per_sm = probe_at(u.probe_wpb);
+            ok = u.probe_per_sm > 0;
+        } else {
+            ok = pick_block(probe_at, u.probe_wpb, u.probe_per_sm);
+        }
+        if (ok) u.probe_per_sm_l = probe_max_blocks_per_sm(V, G, h->eta, PB_LANES, u.probe_wpb, 0);
+        if (!ok || u.probe_per_sm_l < 1) u.set.qw = 0;
+        u.probe_per_sm = std::min(u.probe_per_sm, most);
+        u.probe_per_sm_l = std::min(u.probe_per_sm_l, most);
+        if (ok && group != 1 && u.probe_wpb > 1)
+            u.probe_per_sm_g = std::min(most, probe_max_blocks_per_sm(V, G, h->eta, PB_GROUP, u.probe_wpb,
+                                                                      probe_group_smem_bytes(h->R, h->S, u.probe_wpb)));
+    }
+    h->tuned = u;
+    h->tuned_cfg = h->cfg;
+    h->tuned_known = true;
+    return RAMBO_OK;
+}
+
+// Queries a warp takes per work-queue ticket.
+int ticket_batch(uint64_t n, uint64_t warps) {
+    const uint64_t batch = n / (warps * 32);
+    return (int)(batch < 1 ? 1 : batch > 16 ? 16 : batch);
+}
+
 int resolve_tuning(rambo* h, uint64_t n, int& use_bitmap, QueryTuning& t) {
     t = QueryTuning{};
     if (query_is_wide(h->R, h->S)) {
@@ -538,69 +621,88 @@ int resolve_tuning(rambo* h, uint64_t n, int& use_bitmap, QueryTuning& t) {
     }
     t.V = (int)h->cfg.words_per_lane;
     t.G = (int)h->cfg.lanes_per_key;
-    t.warps_per_block = (int)h->cfg.warps_per_block;
     t.set_stage = (int)h->cfg.set_stage;
     t.order = (int)h->cfg.visit_order;
     t.load_kind = (int)h->cfg.row_load;
     t.staging = h->cfg.answer_staging;
     t.group = (int)h->cfg.warps_per_query;
     use_bitmap = (h->mem_off && t.set_stage != 1 && (h->K + 31) / 32 <= 4096) ? 1 : 0;
-    const size_t spw_bytes = (size_t)query_smem_words_per_warp(h->R, h->S, h->K, use_bitmap) * 4;
-    int per_sm = 0;
-    if (t.warps_per_block == 0) {
-        // The largest block that keeps at least 85% of the most warps any
-        // block size can keep resident per SM.  The per-warp bitmap grows
-        // with K, so for large ID spaces shared memory, not registers, limits
-        // the residency and smaller blocks pack the SM more fully.
-        const int key = (t.V * 64 + t.G) * 2 + use_bitmap;
-        if (h->auto_key != key) {
-            int nb_of[4] = {0, 0, 0, 0}, best = 0;
-            for (int i = 0; i < 4; ++i) {
-                const int w = 8 >> i;
-                nb_of[i] = query_max_blocks_per_sm(t.V, t.G, h->eta, false, w, spw_bytes * (size_t)w);
-                if (nb_of[i] * w > best) best = nb_of[i] * w;
-            }
-            if (best < 1) return RAMBO_EINVAL;
-            for (int i = 0; i < 4; ++i)
-                if (nb_of[i] > 0 && 100 * nb_of[i] * (8 >> i) >= 85 * best) {
-                    h->auto_wpb = 8 >> i;
-                    h->auto_per_sm = nb_of[i];
-                    break;
-                }
-            h->auto_key = key;
-        }
-        t.warps_per_block = h->auto_wpb;
-        per_sm = h->auto_per_sm;
-    } else {
-        per_sm = query_max_blocks_per_sm(t.V, t.G, h->eta, false, t.warps_per_block,
-                                         spw_bytes * (size_t)t.warps_per_block);
-    }
-    if (per_sm < 1) return RAMBO_EINVAL;
-    if (h->cfg.blocks_per_sm && (int)h->cfg.blocks_per_sm < per_sm) per_sm = (int)h->cfg.blocks_per_sm;
-    uint64_t blocks = (uint64_t)per_sm * h->num_sms;
+    if (!h->tuned_known || std::memcmp(&h->tuned_cfg, &h->cfg, sizeof(h->cfg)) != 0) RK(resolve_residency(h, use_bitmap));
+    const rambo::Tuned& u = h->tuned;
+    t.warps_per_block = u.wpb;
+    uint64_t blocks = (uint64_t)u.per_sm * h->num_sms;
     uint64_t need = (n + t.warps_per_block - 1) / t.warps_per_block;
     if (blocks > need) blocks = need;
     if (blocks < 1) blocks = 1;
     t.blocks = (int)blocks;
     // grouped instance (several warps per query): up to one block a query
-    t.blocks_group = 0;
-    t.group_warps = 0;
-    if (use_bitmap && t.group != 1 && t.warps_per_block > 1) {
-        int per_sm_g = query_max_blocks_per_sm(t.V, t.G, h->eta, true, t.warps_per_block,
-                                               query_group_smem_bytes(h->R, h->S, h->K, t.warps_per_block, t.group));
-        if (h->cfg.blocks_per_sm && (int)h->cfg.blocks_per_sm < per_sm_g) per_sm_g = (int)h->cfg.blocks_per_sm;
-        uint64_t bg = (uint64_t)per_sm_g * h->num_sms;
+    uint64_t bg = (uint64_t)u.per_sm_g * h->num_sms;
+    if (bg > n) bg = n;
+    t.blocks_group = (int)bg;
+    t.group_warps = bg * (uint64_t)t.warps_per_block;
+    t.batch = ticket_batch(n, blocks * t.warps_per_block);
+    if (u.set.qw) {
+        t.set = u.set;
+        t.probe_warps = u.probe_wpb;
+        blocks = (uint64_t)u.probe_per_sm * h->num_sms;
+        need = (n + t.probe_warps - 1) / t.probe_warps;
+        t.probe_blocks = (int)(blocks < need ? blocks : need);
+        bg = (uint64_t)u.probe_per_sm_g * h->num_sms;
         if (bg > n) bg = n;
-        if (bg >= 1) {
-            t.blocks_group = (int)bg;
-            t.group_warps = bg * (uint64_t)t.warps_per_block;
-        }
+        t.probe_blocks_group = (int)bg;
+        t.probe_group_warps = bg * (uint64_t)t.probe_warps;
+        // (a warp of the lane-group instance has 32 / G queries in flight)
+        blocks = (uint64_t)u.probe_per_sm_l * h->num_sms;
+        need = (n + (uint64_t)t.probe_warps * 32 / t.G - 1) / ((uint64_t)t.probe_warps * 32 / t.G);
+        t.probe_blocks_lanes = (int)(blocks < need ? blocks : need);
+        t.probe_batch = ticket_batch(n, (uint64_t)t.probe_blocks * t.probe_warps);
     }
-    uint64_t warps = blocks * t.warps_per_block;
-    uint64_t batch = n / (warps * 32);
-    if (batch < 1) batch = 1;
-    if (batch > 16) batch = 16;
-    t.batch = (int)batch;
+    return RAMBO_OK;
+}
+
+// Batches with at most this many bitmap words in all stay with the query
+// kernel, whose blocks then have next to no set stage: the second kernel's
+// launch costs more than it saves (a query over 1e4 sets: 10.9 us in one
+// kernel, 16.0 in two; 16 queries over 1e5 sets: 202 against 28).
+constexpr uint64_t PROBE_LEAST_WORDS = 1024;
+
+// Room for an n-query batch on the probe path: a bitmap a query in the
+// staging arena (grown by at most a quarter of the free memory), and masks
+// and indexes of the queries handed over.  False (the query kernel then
+// answers the batch alone) for the smallest batches, when the tuning asks for
+// a set stage or staging form of the query kernel, or when memory is short.
+bool probe_room(rambo* h, uint64_t n, const QueryTuning& t) {
+    if (!t.set.qw || n > 0xffffffffull || n * ((h->K + 31) / 32) <= PROBE_LEAST_WORDS) return false;
+    const uint64_t pitch = set_pitch(h->K);
+    if (h->stage.cap / pitch < n) {
+        size_t free_b = 0, total_b = 0;
+        if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || (uint64_t)free_b / 16 / pitch < n) {
+            cudaGetLastError();
+            return false;
+        }
+        if (h->stage.ensure(n * pitch) != RAMBO_OK) return false;
+    }
+    return h->dmask.ensure(n * h->R * h->S) == RAMBO_OK && h->dq.ensure(2 * n) == RAMBO_OK;
+}
+
+// The queries' answers staged and counted (o.dmask set: probe and set kernel,
+// else the query kernel alone), and the counts scanned into CSR offsets.
+int enqueue_answers(rambo* h, const BatchView& b, const QueryOut& o, const QueryTuning& t, int use_bitmap,
+                    uint64_t* d_off, const uint64_t* base_dev, cudaEvent_t staged, cudaStream_t s) {
+    int nl = 0, n_scan = 0;
+    bool scanned = false;
+    if (o.dmask) {
+        CK(launch_probe(h->view(), h->hp, b, o, t, h->st, s, &nl));
+        scanned = b.n <= SET_SCAN_MAX;
+        CK(launch_set(t.set, h->view(), b, o, scanned, d_off, base_dev, nullptr, h->st, s));
+        ++nl;
+    } else {
+        CK(launch_query(h->view(), h->hp, b, o, t, use_bitmap, h->st, s, &nl));
+    }
+    if (staged) CK(cudaEventRecord(staged, s));
+    if (!scanned)
+        CK(launch_scan_counts(o.qcount, b.n, d_off, h->scan_tmp.p, h->scan_tmp.cap, s, nullptr, &n_scan, base_dev));
+    h->launches += (uint64_t)(nl + n_scan);
     return RAMBO_OK;
 }
 
@@ -667,6 +769,10 @@ int run_query_pipelined(rambo* h, BatchView b, const void* d_data, int seq, uint
     const int C = h->cfg.host_chunks ? (int)h->cfg.host_chunks : 4;
     uint64_t q_lo[PIPE_MAX_CHUNKS + 1];
     for (int c = 0; c <= C; ++c) q_lo[c] = n * (uint64_t)c / (uint64_t)C;
+    int ub0 = 0;
+    QueryTuning t0{};
+    RK(resolve_tuning(h, n, ub0, t0));
+    const bool probe = probe_room(h, n / (uint64_t)C + 1, t0);
 
     CK(cudaEventRecord(h->ev[0], s));
     RK(enqueue_intake(h, b, d_data, seq, k, s));
@@ -690,22 +796,19 @@ int run_query_pipelined(rambo* h, BatchView b, const void* d_data, int seq, uint
         int ub = 0;
         QueryTuning t{};
         RK(resolve_tuning(h, nc, ub, t));
-        QueryOut oc{h->stage.p, h->stage.cap, h->qstart.p + q_lo[c], h->qcount.p + q_lo[c], 0, 0};
+        QueryOut oc{h->stage.p, h->stage.cap, h->qstart.p + q_lo[c], h->qcount.p + q_lo[c]};
         set_staging(oc, h->K, h->cfg.answer_staging);
-        if (c) {  // fresh work queues for the chunk's query and gather kernels
-            CK(cudaMemsetAsync(&h->st->ticket, 0, sizeof(unsigned long long), s));
-            CK(cudaMemsetAsync(&h->st->gather_ticket, 0, sizeof(unsigned long long), s));
-        }
-        int nl = 0, n_scan = 0;
-        CK(launch_query(h->view(), h->hp, bc, oc, t, ub, h->st, s, &nl));
+        // (a chunk's bitmaps and masks are used up before the next chunk's are written)
+        if (probe) oc.dmask = h->dmask.p, oc.dq = h->dq.p, oc.dlong = h->dq.p + h->dq.cap / 2;
+        // fresh work queues for the chunk's kernels
+        if (c) CK(cudaMemsetAsync(&h->st->ticket, 0, QUEUE_BYTES, s));
         // chunk c's offsets continue from the total written by chunk c - 1's scan
         if (c) CK(cudaMemcpyAsync(h->pslot.p + c, d_off + q_lo[c], sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));
-        CK(launch_scan_counts(oc.qcount, nc, d_off + q_lo[c], h->scan_tmp.p, h->scan_tmp.cap, s, nullptr, &n_scan,
-                              h->pslot.p + c));
+        RK(enqueue_answers(h, bc, oc, t, ub, d_off + q_lo[c], h->pslot.p + c, nullptr, s));
         CK(launch_gather(oc, d_off + q_lo[c], nc, h->ids.p, h->st, s, nullptr, cap));
         CK(cudaMemcpyAsync(h->ptot.p + c, d_off + q_lo[c + 1], sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
         CK(cudaEventRecord(h->pev[c], s));
-        h->launches += (uint64_t)(nl + n_scan + 1);
+        h->launches += 1;
     }
     CK(cudaEventRecord(h->ev[2], s));
     CK(cudaMemcpyAsync(h->pst.p + 1, h->st, sizeof(DevStatus), cudaMemcpyDeviceToHost, s));
@@ -745,7 +848,7 @@ int run_query_pipelined(rambo* h, BatchView b, const void* d_data, int seq, uint
     h->last.rows_read = fin.rows_read;
     h->last.n_results = prev;
     for (int i = 0; i < 4; ++i) h->last.stage_queries[i] = fin.stage_count[i];
-    h->last.staged_words = fin.cursor;
+    h->last.staged_words = probe ? fin.spare[0] : fin.cursor;
     // (the chunks' query kernels, interleaved with their scans and gathers)
     CK(cudaEventElapsedTime(&h->last.query_kernel_ms, h->ev[1], h->ev[2]));
     CK(cudaEventElapsedTime(&h->last.device_ms, h->ev[0], h->ev[3]));
@@ -802,7 +905,8 @@ int run_query(rambo* h, int seq, const void* data, const uint64_t* offsets, uint
     RK(h->qcount.ensure(n));
     RK(h->qstart.ensure(n));
     RK(h->scan_tmp.ensure(scan_tmp_words(n)));
-    if (h->stage.cap < (1u << 20)) RK(h->stage.ensure(1u << 20));
+    const bool probe = probe_room(h, n, t);
+    if (!probe && h->stage.cap < (1u << 20)) RK(h->stage.ensure(1u << 20));
     if (!on_device && d.arena && n >= PIPE_MIN_QUERIES && !h->cfg.cluster && !h->cfg.l2_fetch_bytes &&
         h->cfg.host_chunks != 1) {
         const int rc = run_query_pipelined(h, b, d_data, seq, k, n, s, d);
@@ -832,20 +936,17 @@ int run_query(rambo* h, int seq, const void* data, const uint64_t* offsets, uint
             b.perm = h->perm.p;
             h->launches += 5;
         }
-        QueryOut o{h->stage.p, h->stage.cap, h->qstart.p, h->qcount.p, 0, 0};
+        QueryOut o{h->stage.p, h->stage.cap, h->qstart.p, h->qcount.p};
         set_staging(o, h->K, h->cfg.answer_staging);
+        if (probe) o.dmask = h->dmask.p, o.dq = h->dq.p, o.dlong = h->dq.p + h->dq.cap / 2;
         size_t l2_prev = 0;
         if (h->cfg.l2_fetch_bytes) {
             CK(cudaDeviceGetLimit(&l2_prev, cudaLimitMaxL2FetchGranularity));
             CK(cudaDeviceSetLimit(cudaLimitMaxL2FetchGranularity, h->cfg.l2_fetch_bytes));
         }
         CK(cudaEventRecord(h->ev[1], s));
-        CK(launch_query(h->view(), h->hp, b, o, t, use_bitmap, h->st, s));
-        CK(cudaEventRecord(h->ev[2], s));
+        RK(enqueue_answers(h, b, o, t, use_bitmap, d_off, nullptr, h->ev[2], s));
         if (h->cfg.l2_fetch_bytes) CK(cudaDeviceSetLimit(cudaLimitMaxL2FetchGranularity, l2_prev));
-        int n_scan = 0;
-        CK(launch_scan_counts(h->qcount.p, n, d_off, h->scan_tmp.p, h->scan_tmp.cap, s, nullptr, &n_scan));
-        h->launches += 1 + n_scan;
         CK(cudaMemcpyAsync(h->h_st, h->st, sizeof(DevStatus), cudaMemcpyDeviceToHost, s));
         CK(cudaMemcpyAsync(h->h_small, d_off + n, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
@@ -865,7 +966,7 @@ int run_query(rambo* h, int seq, const void* data, const uint64_t* offsets, uint
     CK(cudaEventElapsedTime(&h->last.query_kernel_ms, h->ev[1], h->ev[2]));
     if (d.needed) *d.needed = total_ids;
     if (!d.arena && total_ids > d.ids_cap) return RAMBO_ENOSPC;
-    QueryOut o{h->stage.p, h->stage.cap, h->qstart.p, h->qcount.p, 0, 0};
+    QueryOut o{h->stage.p, h->stage.cap, h->qstart.p, h->qcount.p};
     set_staging(o, h->K, h->cfg.answer_staging);
     if (on_device) {
         uint32_t* d_ids;

@@ -35,14 +35,20 @@ constexpr unsigned PRIO_EBADSEQ = 3;
 struct DevStatus {
     unsigned long long err;          // see above; NO_ERR when clean
     unsigned long long bad_pos;      // lowest position of a byte outside ACGTacgt
-    unsigned long long ticket;       // next query index handed out to a warp
+    // work queues, cleared together between the chunks of a host-output batch
+    unsigned long long ticket;         // next query index handed out to a warp
+    unsigned long long gather_ticket;  // next queries handed out to a gather warp
+    unsigned long long n_handed;       // queries the probe kernel handed to the set kernel
+    unsigned long long set_done;       // finished blocks of the set kernel
+    unsigned long long n_long;         // long queries of a batch of short ones (see k_probe.cuh)
+    unsigned long long ticket_long;    // next of them handed out to a warp
     unsigned long long cursor;       // staged result IDs handed out so far
     unsigned long long keys_probed;  // keys whose rows were read
     unsigned long long rows_read;    // row reads issued
     unsigned long long spare[2];
     unsigned long long stage_count[4];   // surviving queries per set stage (1 dense, 2 sparse, 3 union)
-    unsigned long long gather_ticket;    // next queries handed out to a gather warp
 };
+constexpr size_t QUEUE_BYTES = 6 * sizeof(unsigned long long);  // ticket .. ticket_long
 
 // Position multipliers s_{r,j}, passed by value so every warp reads them from
 // the kernel-parameter bank (uniform across the warp).
@@ -301,7 +307,16 @@ struct QueryOut {
     uint32_t* qcount;      // per query: number of IDs
     uint32_t bits_words;   // ceil(K/32) when bitmap staging is allowed, else 0
     uint32_t bits_min;     // an answer of more IDs than this is staged as the bitmap
+    // set on the probe path (k_probe.cuh): what it hands to the set kernel,
+    // in the order queries were handed over; slot i's bitmap is staged at
+    // word i * set_pitch(K)
+    uint32_t* dmask;       // [n][R * S] per-table cell masks
+    uint32_t* dq;          // [n] query index
+    uint32_t* dlong;       // [n] long queries of a batch of short ones
 };
+
+// Words of a bitmap staged for the set kernel: whole groups of 256 IDs.
+__host__ __device__ inline uint64_t set_pitch(uint64_t K) { return (K + 255) / 256 * 8; }
 
 // Staging form for an ID space of K sets: staging 0 = bitmap above ceil(K/32)
 // IDs, 1 = ID lists only, f >= 2 = bitmap above f * ceil(K/32) IDs.  A query
@@ -317,6 +332,13 @@ inline void set_staging(QueryOut& o, uint64_t K, uint32_t staging) {
     o.bits_min = m > 0xffffffffull ? 0xffffffffu : (uint32_t)m;
 }
 
+// The set kernel's launch (k_query_set.cu).
+struct SetLaunch {
+    int qw;        // words of queries per cell (32 * qw queries at a time); 0 = this index is not served
+    size_t smem;
+    int blocks;    // one resident wave
+};
+
 struct QueryTuning {
     int V, G;              // words per lane, lanes per key
     int warps_per_block;
@@ -330,6 +352,10 @@ struct QueryTuning {
     unsigned long long group_warps;  // its warps, the budget the group size is chosen against
     int wide;              // 1: the block-per-query kernel (R > RF or rows wider than FAST_MAX_S words)
     uint32_t staging;      // answer staging form (see set_staging)
+    SetLaunch set;         // the set kernel's launch (qw = 0: this tuning keeps the set stage in the query kernel)
+    int probe_warps, probe_batch;  // the probe kernel's counterparts
+    int probe_blocks, probe_blocks_group, probe_blocks_lanes;
+    unsigned long long probe_group_warps;
 };
 
 // ---------------------------------------------------------------------------
@@ -397,6 +423,21 @@ unsigned query_group_size(uint64_t n, int group, unsigned wpb, uint64_t group_wa
 cudaError_t launch_query(const IndexView& ix, const HashParams& hp, const BatchView& b, const QueryOut& o,
                          const QueryTuning& t, int use_bitmap, DevStatus* st, cudaStream_t s,
                          int* n_launched = nullptr);
+
+// k_probe*.cu: the probes of a batch whose set stage the set kernel runs
+constexpr int PB_WARP = 0, PB_GROUP = 1, PB_LANES = 2;  // its instances
+size_t probe_group_smem_bytes(uint32_t R, uint32_t S, int wpb);
+int probe_max_blocks_per_sm(int V, int G, uint32_t eta, int mode, int warps_per_block, size_t smem);
+cudaError_t launch_probe(const IndexView& ix, const HashParams& hp, const BatchView& b, const QueryOut& o,
+                         const QueryTuning& t, DevStatus* st, cudaStream_t s, int* n_launched);
+
+// k_query_set.cu: the set stage of the queries handed over, 32 to 128 of them
+// at a time, and (scan != 0) the exclusive scan of the counts
+SetLaunch set_launch_shape(const IndexView& ix, int num_sms);
+constexpr uint64_t SET_SCAN_MAX = 32768;  // queries whose counts the set kernel scans itself
+cudaError_t launch_set(const SetLaunch& sl, const IndexView& ix, const BatchView& b, const QueryOut& o, int scan,
+                       uint64_t* id_offsets, const uint64_t* base_dev, unsigned long long* total_out, DevStatus* st,
+                       cudaStream_t s);
 
 // k_query_wide.cu: block-per-query kernel for wide rows or many tables
 constexpr int QW_THREADS = 256;

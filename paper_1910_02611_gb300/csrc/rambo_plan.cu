@@ -61,6 +61,9 @@ struct rambo_plan {
     uint64_t* qstart = nullptr;
     uint64_t* scan_tmp = nullptr;
     uint32_t* stage = nullptr;
+    uint32_t* dmask = nullptr;  // masks and indexes of the queries handed to the set kernel
+    uint32_t* dq = nullptr;
+    bool probe = false;
     uint32_t* ids = nullptr;
     uint64_t* id_off = nullptr;
     PlanHead* d_head = nullptr;
@@ -108,7 +111,7 @@ void plan_free(rambo_plan* p) {
         if (e) cudaEventDestroy(e);
     if (p->cap) cudaStreamDestroy(p->cap);
     void* dev[] = {p->d_data, p->d_off, p->d_packed, p->d_nmask, p->qcount, p->qstart, p->scan_tmp,
-                   p->stage, p->ids, p->id_off, p->d_head};
+                   p->stage, p->dmask, p->dq, p->ids, p->id_off, p->d_head};
     for (void* d : dev)
         if (d) cudaFree(d);
     void* host[] = {p->h_data, p->h_off, p->h_head, p->h_st, p->h_ids, p->h_id_off};
@@ -155,16 +158,20 @@ int plan_capture(rambo_plan* p, bool timed) {
                           p->kind == 1 ? p->max_items / 32 + 2 : 0, p->d_nmask, p->st, s),
         ++n_launch;
     if (e == cudaSuccess && p->kind == 1 && p->skipn) e = launch_check_windows(b, p->st, s), ++n_launch;
-    QueryOut o{p->stage, p->stage_words, p->qstart, p->qcount, 0, 0};
+    QueryOut o{p->stage, p->stage_words, p->qstart, p->qcount};
     set_staging(o, ix.K, p->staging);
+    if (p->probe) o.dmask = p->dmask, o.dq = p->dq, o.dlong = p->dq + p->max_q;
     if (e == cudaSuccess) e = mark(p, 1, s, timed);
     if (e == cudaSuccess) {
         int nq = 0;
-        e = launch_query(ix, hp, b, o, t, use_bitmap, p->st, s, &nq);
+        e = p->probe ? launch_probe(ix, hp, b, o, t, p->st, s, &nq) : launch_query(ix, hp, b, o, t, use_bitmap, p->st, s, &nq);
         n_launch += nq;
     }
+    const bool scanned = p->probe && p->max_q <= SET_SCAN_MAX;  // the set kernel also scans the counts
+    if (e == cudaSuccess && p->probe)
+        e = launch_set(t.set, ix, b, o, scanned, p->id_off, nullptr, &p->st->spare[1], p->st, s), ++n_launch;
     if (e == cudaSuccess) e = mark(p, 2, s, timed);
-    if (e == cudaSuccess) {
+    if (e == cudaSuccess && !scanned) {
         int n_scan = 0;
         // the scan also stores the number of result IDs in the status block
         e = launch_scan_counts(p->qcount, p->max_q, p->id_off, p->scan_tmp, scan_words, s, p->d_desc, &n_scan,
@@ -252,6 +259,26 @@ int rambo_plan_create(rambo_t* h, int kind, uint64_t max_queries, uint64_t max_i
         set_staging(form, ix.K, t.staging);
         if (form.bits_words && max_queries <= max_ids / form.bits_min) p->stage_words = max_queries * form.bits_min;
     }
+    // On the probe path every answer is staged as a bitmap of set_pitch(K)
+    // words.  It is taken when an arena for max_queries of them is no more
+    // than four times the one above, or 256 MiB, and memory holds it.
+    const uint64_t pitch = set_pitch(ix.K), plain_words = p->stage_words;
+    const uint64_t most = plain_words * 4 > (64ull << 20) ? plain_words * 4 : 64ull << 20;
+    if (t.set.qw && max_queries <= most / pitch) {
+        const uint64_t words = max_queries * pitch;
+        p->probe = cudaSetDevice(p->device) == cudaSuccess && cudaMalloc(&p->stage, words * 4) == cudaSuccess &&
+                   cudaMalloc(&p->dmask, max_queries * ix.R * ix.S * 4) == cudaSuccess &&
+                   cudaMalloc(&p->dq, max_queries * 8) == cudaSuccess;
+        if (p->probe) {
+            p->stage_words = words;
+        } else {
+            cudaGetLastError();
+            for (uint32_t** d : {&p->stage, &p->dmask, &p->dq}) {
+                if (*d) cudaFree(*d);
+                *d = nullptr;
+            }
+        }
+    }
     p->elem = kind == 0 ? 8 : 1;
     auto fail = [&](int code) {
         plan_free(p);
@@ -265,7 +292,7 @@ int rambo_plan_create(rambo_t* h, int kind, uint64_t max_queries, uint64_t max_i
               cudaMalloc(&p->qcount, max_queries * 4) == cudaSuccess &&
               cudaMalloc(&p->qstart, max_queries * 8) == cudaSuccess &&
               cudaMalloc(&p->scan_tmp, scan_tmp_words(max_queries) * 8) == cudaSuccess &&
-              cudaMalloc(&p->stage, p->stage_words * 4) == cudaSuccess && cudaMalloc(&p->ids, max_ids * 4) == cudaSuccess &&
+              (p->stage || cudaMalloc(&p->stage, p->stage_words * 4) == cudaSuccess) && cudaMalloc(&p->ids, max_ids * 4) == cudaSuccess &&
               cudaMalloc(&p->id_off, (max_queries + 1) * 8) == cudaSuccess &&
               cudaMalloc(&p->d_head, sizeof(PlanHead)) == cudaSuccess &&
               cudaMallocHost(&p->h_data, max_items * p->elem + 16) == cudaSuccess &&
