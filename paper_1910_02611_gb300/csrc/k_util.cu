@@ -2,6 +2,8 @@
 // 2-bit packing (batch intake), set registration, the partition table and its
 // per-cell member lists, the count scan and result gather of the compaction
 // step, and index statistics.
+#include <algorithm>
+
 #include "rambo_impl.cuh"
 
 namespace rgb {
@@ -548,123 +550,217 @@ cudaError_t launch_cluster_order(const BatchView& b, uint64_t* keys, uint32_t* h
 }
 
 // ---------------------------------------------------------------------------
-// gather staged result IDs into CSR order: one warp per query, warps taking
-// GA_TAKE queries at a time from a work queue (answers range from nothing to
-// the whole ID space, so a fixed share per warp would leave a long tail).  A
-// query staged as its K-bit bitmap is expanded 32 words (up to 1024 IDs) at a
-// time: every lane writes its word's set bits as IDs into the warp's run in
-// shared memory at its prefix position, then the warp stores the run with
-// coalesced writes (32 full words need no run: their IDs are consecutive).  The prefix of the lanes' bit counts (0..32, six bits)
-// comes from six ballots, one per bit of the count, instead of a chain of
-// shuffles.
+// gather staged result IDs into CSR order.  Answers range from nothing to the
+// whole ID space, so warps take them from a work queue, and a long answer
+// staged as a bitmap is cut into parts for several warps (one warp took 330
+// us for 1e5 IDs, which was the whole kernel for a batch of a few hundred
+// queries and the tail of a larger one).  A part starts where the set bits
+// before it end: its warp counts them, 32 words and some four instructions at
+// a time, against some ten a word to expand.
+//
+// What bounds it: instruction issue where answers are dense (a bit test and a
+// shared store for every bit position), the writes of the IDs otherwise.
+// Measured, one warp per answer -> parts: 16 queries over 1e5 documents (3e5
+// IDs) 177 -> about 50 us, 256 of them (5e6) 335 -> 57 us, 1e4 over 5e5
+// documents (9.8e8 IDs; staged as lists before) 11.8 -> 0.93 ms, 1e5 over 1e5
+// (2e9 IDs, 8 GB) 1.76 -> 1.65 ms.  Parts of 2048 words: 4096 measured 5%
+// slower on the last of these, 512 and 1024 slower on the one before it.
+//
+// A query staged as its K-bit bitmap is expanded 32 words (up to 1024 IDs) at
+// a time: every lane writes its word's set bits as IDs into the warp's run in
+// shared memory at its prefix position, then the warp stores the run 16 bytes
+// a lane (32 full words need no run: their IDs are consecutive).  The prefix
+// of the lanes' bit counts (0..32, six bits) comes from six ballots, one per
+// bit of the count, instead of a chain of shuffles.
 
 constexpr int GA_THREADS = 256;
-constexpr int GA_RUN = 1024;  // IDs of 32 bitmap words
-constexpr int GA_RUN_PAD = GA_RUN + GA_RUN / 32;  // the run with one pad word per 32
-constexpr unsigned GA_TAKE = 8;  // queries per work-queue ticket
+constexpr int GA_WARPS = GA_THREADS / 32;
+constexpr int GA_RUN = 1024;                  // IDs of 32 bitmap words
+constexpr uint32_t GA_SHORT = 4096;           // answers of at most this many IDs are not cut
+constexpr uint32_t GA_PART_WORDS = 2048;     // bitmap words of a part in a batch that fills the grid,
+constexpr uint32_t GA_PART_LEAST = 128;       // and of the smallest part where it does not
+constexpr unsigned GA_TAKE = 8;               // most parts per work-queue ticket
 
-__global__ void __launch_bounds__(GA_THREADS) k_gather(QueryOut o, const uint64_t* __restrict__ id_offsets, uint64_t n,
+// entry p of a run: four pad words per 32, so lanes whose words are all full
+// do not store to one bank, and four entries from a multiple of four stay
+// 16-byte aligned
+__device__ __forceinline__ uint32_t ga_at(uint32_t p) { return p + (p >> 5) * 4; }
+constexpr int GA_RUN_WORDS = (GA_RUN + 4) + (GA_RUN + 4) / 32 * 4 + 4;
+
+// Stores n IDs at dst, 16 bytes a lane and step: entry i of the answer is
+// value(ph + i) where ph is dst's word offset in its 16 bytes.
+template <class F>
+__device__ __forceinline__ void ga_store(uint32_t* dst, uint32_t n, unsigned lane, F four) {
+    const uint32_t ph = (uint32_t)(reinterpret_cast<uintptr_t>(dst) >> 2) & 3u;
+    uint32_t* base = dst - ph;
+    const uint32_t end = ph + n;
+    for (uint32_t i = lane * 4; i < end; i += 128) {
+        const uint4 x = four(i);
+        if (i >= ph && i + 4 <= end) {
+            *reinterpret_cast<uint4*>(base + i) = x;
+        } else {
+            if (i >= ph && i < end) base[i] = x.x;
+            if (i + 1 >= ph && i + 1 < end) base[i + 1] = x.y;
+            if (i + 2 >= ph && i + 2 < end) base[i + 2] = x.z;
+            if (i + 3 >= ph && i + 3 < end) base[i + 3] = x.w;
+        }
+    }
+}
+
+// One warp expands words [w_lo, w_hi) of a bitmap into IDs at dst.  The words
+// of the next two steps are loaded ahead, so their latency overlaps this one.
+__device__ __forceinline__ void ga_expand(const uint32_t* __restrict__ src, uint32_t w_lo, uint32_t w_hi,
+                                          uint32_t* __restrict__ dst, uint32_t* run, unsigned lane) {
+    const unsigned lt = (1u << lane) - 1u;  // lanes below this one
+    uint32_t cur = w_lo + lane < w_hi ? __ldcs(src + w_lo + lane) : 0u;
+    uint32_t nx1 = w_lo + 32 + lane < w_hi ? __ldcs(src + w_lo + 32 + lane) : 0u;
+    for (uint32_t w0 = w_lo; w0 < w_hi; w0 += 32) {
+        const uint32_t w = w0 + lane;
+        const uint32_t nx2 = w + 64 < w_hi ? __ldcs(src + w + 64) : 0u;
+        uint32_t bits = cur;
+        cur = nx1;
+        nx1 = nx2;
+        if (!__any_sync(FULL, bits)) continue;
+        const uint32_t cw = __popc(bits);
+        uint32_t pos = 0, blk = 0;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const unsigned m = __ballot_sync(FULL, (cw >> k) & 1u);
+            pos += (uint32_t)__popc(m & lt) << k;
+            blk += (uint32_t)__popc(m) << k;
+        }
+        const uint32_t ph = (uint32_t)(reinterpret_cast<uintptr_t>(dst) >> 2) & 3u;
+        if (blk == GA_RUN) {
+            // 32 full words: the IDs are consecutive
+            const uint32_t id0 = w0 * 32 - ph;
+            ga_store(dst, blk, lane, [&](uint32_t i) { return make_uint4(id0 + i, id0 + i + 1, id0 + i + 2, id0 + i + 3); });
+            dst += blk;
+            continue;
+        }
+        pos += ph;
+        if (blk > GA_RUN / 2) {
+            // dense words: every bit position in turn, no bit scans
+#pragma unroll
+            for (int b = 0; b < 32; ++b) {
+                const uint32_t on = (bits >> b) & 1u;
+                if (on) run[ga_at(pos)] = w * 32 + b;
+                pos += on;
+            }
+        } else {
+            // (a run of at most half the entries needs no padding: its lanes start apart)
+            for (uint32_t* r = run + pos; bits; bits &= bits - 1) *r++ = w * 32 + (__ffs(bits) - 1);
+        }
+        __syncwarp();
+        if (blk > GA_RUN / 2)
+            ga_store(dst, blk, lane, [&](uint32_t i) { return *reinterpret_cast<const uint4*>(run + ga_at(i)); });
+        else
+            ga_store(dst, blk, lane, [&](uint32_t i) { return *reinterpret_cast<const uint4*>(run + i); });
+        __syncwarp();  // the run is rewritten by the next 32 words
+        dst += blk;
+    }
+}
+
+// Copies n words of an ID list, four independent loads in flight a lane.
+__device__ __forceinline__ void ga_copy(const uint32_t* __restrict__ src, uint32_t n, uint32_t* __restrict__ dst,
+                                        unsigned lane) {
+    uint32_t t = lane;
+    for (; t + 96 < n; t += 128) {
+        const uint32_t a0 = __ldcs(src + t), a1 = __ldcs(src + t + 32);
+        const uint32_t a2 = __ldcs(src + t + 64), a3 = __ldcs(src + t + 96);
+        dst[t] = a0;
+        dst[t + 32] = a1;
+        dst[t + 64] = a2;
+        dst[t + 96] = a3;
+    }
+#pragma unroll 1
+    for (; t < n; t += 32) dst[t] = __ldcs(src + t);
+}
+
+// Set bits of the first `words` words (a multiple of 32): this lane's share of a warp's sum.
+__device__ __forceinline__ uint32_t ga_count(const uint32_t* __restrict__ src, uint32_t words, unsigned lane) {
+    uint32_t c = 0;
+    if (reinterpret_cast<uintptr_t>(src) & 15) {
+#pragma unroll 8
+        for (uint32_t w = lane; w < words; w += 32) c += __popc(__ldg(src + w));
+    } else {
+#pragma unroll 4
+        for (uint32_t w = lane * 4; w < words; w += 128) {
+            const uint4 x = __ldg(reinterpret_cast<const uint4*>(src + w));
+            c += __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w);
+        }
+    }
+    return c;
+}
+
+// Parts a long answer is cut into when n queries share a grid of `warps`.
+__device__ __forceinline__ uint32_t ga_parts(uint32_t bits_words, uint64_t n, uint64_t warps) {
+    const uint32_t base = bits_words ? (bits_words + GA_PART_WORDS - 1) / GA_PART_WORDS : 4;
+    const uint32_t most = bits_words ? (bits_words + GA_PART_LEAST - 1) / GA_PART_LEAST : 16;
+    const uint64_t fill = warps / n;  // parts that occupy every warp
+    const uint32_t parts = fill < most ? (uint32_t)fill : most;
+    return parts > base ? parts : base;
+}
+
+__global__ void __launch_bounds__(GA_THREADS, 6) k_gather(QueryOut o, const uint64_t* __restrict__ id_offsets, uint64_t n,
                                                         uint32_t* __restrict__ ids, DevStatus* st,
                                                         const uint64_t* __restrict__ n_dev, uint64_t ids_cap) {
-    __shared__ uint32_t s_run[GA_THREADS / 32][GA_RUN_PAD];
+    __shared__ __align__(16) uint32_t s_run[GA_WARPS][GA_RUN_WORDS];
     if (st->err != NO_ERR || st->cursor > o.stage_cap) return;
     if (n_dev) n = *n_dev;
-    if (id_offsets[n] > ids_cap) return;  // the caller sees the total and reports the shortfall
+    if (n == 0 || id_offsets[n] > ids_cap) return;  // the caller sees the total and reports the shortfall
     const unsigned lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;  // lanes below this one
     uint32_t* run = s_run[threadIdx.x >> 5];
-    for (;;) {
-        unsigned long long q0 = 0;
-        if (lane == 0) q0 = atomicAdd(&st->gather_ticket, (unsigned long long)GA_TAKE);
-        q0 = __shfl_sync(0xffffffffu, q0, 0);
-        if (q0 >= n) break;
-        const uint64_t q1 = min((unsigned long long)n, q0 + GA_TAKE);
-        for (uint64_t q = q0; q < q1; ++q) {
-            const uint32_t c = o.qcount[q];
-            if (!c) continue;
-            const uint64_t s0 = o.qstart[q];
-            uint32_t* dst = ids + id_offsets[q];
-            if (!(s0 & QSTART_BITMAP)) {
-                // an ID list: four independent loads in flight per lane
-                const uint32_t* src = o.stage + s0;
-                uint32_t t = lane;
-                for (; t + 96 < c; t += 128) {
-                    const uint32_t a0 = __ldcs(src + t), a1 = __ldcs(src + t + 32);
-                    const uint32_t a2 = __ldcs(src + t + 64), a3 = __ldcs(src + t + 96);
-                    dst[t] = a0;
-                    dst[t + 32] = a1;
-                    dst[t + 64] = a2;
-                    dst[t + 96] = a3;
-                }
-                for (; t < c; t += 32) dst[t] = __ldcs(src + t);
-                continue;
-            }
-            // a bitmap, 32 words at a time; the words of the next two steps are
-            // loaded ahead so their latency overlaps the expansion of this one
-            const uint32_t* src = o.stage + (s0 & ~QSTART_BITMAP);
-            const uint32_t bw = o.bits_words;
-            uint32_t cur = lane < bw ? __ldcs(src + lane) : 0u;
-            uint32_t nx1 = 32 + lane < bw ? __ldcs(src + 32 + lane) : 0u;
-            uint32_t at = 0;
-            for (uint32_t w0 = 0; w0 < bw; w0 += 32) {
-                const uint32_t w = w0 + lane;
-                const uint32_t nx2 = w + 64 < bw ? __ldcs(src + w + 64) : 0u;
-                uint32_t bits = cur;
-                cur = nx1;
-                nx1 = nx2;
-                const uint32_t cw = __popc(bits);
-                uint32_t pos = 0, blk = 0;
-#pragma unroll
-                for (int k = 0; k < 6; ++k) {
-                    const unsigned m = __ballot_sync(0xffffffffu, (cw >> k) & 1u);
-                    pos += (uint32_t)__popc(m & lt) << k;
-                    blk += (uint32_t)__popc(m) << k;
-                }
-                if (blk == GA_RUN) {
-                    // 32 full words: the IDs are consecutive
-                    for (uint32_t t = lane; t < GA_RUN; t += 32) dst[at + t] = w0 * 32 + t;
-                    at += blk;
-                    continue;
-                }
-                // the run is padded by one word per 32 (entry p at p + p/32), so
-                // lanes whose words are full do not all write one bank
-                if (blk > GA_RUN / 2) {
-                    // dense words: every bit position in turn, no bit scans
-#pragma unroll
-                    for (int b = 0; b < 32; ++b) {
-                        const uint32_t on = (bits >> b) & 1u;
-                        if (on) run[pos + (pos >> 5)] = w * 32 + b;
-                        pos += on;
-                    }
-                } else {
-                    while (bits) {
-                        run[pos + (pos >> 5)] = w * 32 + (__ffs(bits) - 1);
-                        ++pos;
-                        bits &= bits - 1;
-                    }
-                }
-                __syncwarp();
-                uint32_t t = lane;
-                for (; t + 96 < blk; t += 128) {
-                    const uint32_t a0 = run[t + (t >> 5)], a1 = run[t + 32 + ((t + 32) >> 5)];
-                    const uint32_t a2 = run[t + 64 + ((t + 64) >> 5)], a3 = run[t + 96 + ((t + 96) >> 5)];
-                    dst[at + t] = a0;
-                    dst[at + t + 32] = a1;
-                    dst[at + t + 64] = a2;
-                    dst[at + t + 96] = a3;
-                }
-                for (; t < blk; t += 32) dst[at + t] = run[t + (t >> 5)];
-                __syncwarp();  // the run is rewritten by the next 32 words
-                at += blk;
+    const uint64_t warps = (uint64_t)gridDim.x * GA_WARPS;
+    const uint32_t parts = ga_parts(o.bits_words, n, warps);
+    const uint64_t units = n * parts;
+    // answers that are cut into many parts are taken a part at a time, so that
+    // a long one's parts go to several warps; the first take needs no ticket
+    const unsigned take = parts == 1 ? GA_TAKE : parts < 8 && units >= warps * GA_TAKE ? GA_TAKE / 2 : 1;
+    for (unsigned long long u0 = ((uint64_t)blockIdx.x * GA_WARPS + (threadIdx.x >> 5)) * take; u0 < units;) {
+        // a lane looks up each unit of the ticket, then the warp takes them one by one
+        uint32_t c_of = 0, part_of = 0;
+        uint64_t s_of = 0, d_of = 0;
+        const uint64_t mine = u0 + lane;
+        if (lane < take && mine < units) {
+            const uint64_t q = parts == 1 ? mine : mine / parts;
+            part_of = (uint32_t)(mine - q * parts);
+            c_of = o.qcount[q];
+            if (part_of && c_of <= GA_SHORT) c_of = 0;
+            if (c_of) {
+                s_of = o.qstart[q];
+                d_of = id_offsets[q];
             }
         }
+        for (unsigned todo = __ballot_sync(FULL, c_of != 0); todo; todo &= todo - 1) {
+            const int l = __ffs(todo) - 1;
+            const uint32_t c = __shfl_sync(FULL, c_of, l), part = __shfl_sync(FULL, part_of, l);
+            const uint64_t s0 = __shfl_sync(FULL, s_of, l);
+            uint32_t* dst = ids + __shfl_sync(FULL, d_of, l);
+            if (!(s0 & QSTART_BITMAP)) {
+                const uint32_t p = c > GA_SHORT ? parts : 1;
+                const uint32_t lo = (uint32_t)((uint64_t)c * part / p), hi = (uint32_t)((uint64_t)c * (part + 1) / p);
+                ga_copy(o.stage + s0 + lo, hi - lo, dst + lo, lane);
+                continue;
+            }
+            const uint32_t* src = o.stage + (s0 & ~QSTART_BITMAP);
+            uint32_t w_lo = 0, w_hi = o.bits_words;
+            if (parts > 1 && c > GA_SHORT) {
+                const uint32_t groups = (o.bits_words + 31) / 32;
+                w_lo = (uint32_t)((uint64_t)groups * part / parts) * 32;
+                w_hi = min(w_hi, (uint32_t)((uint64_t)groups * (part + 1) / parts) * 32);
+                dst += __reduce_add_sync(FULL, ga_count(src, w_lo, lane));
+            }
+            ga_expand(src, w_lo, w_hi, dst, run, lane);
+        }
+        if (lane == 0) u0 = warps * take + atomicAdd(&st->gather_ticket, (unsigned long long)take);
+        u0 = __shfl_sync(FULL, u0, 0);
     }
 }
 
 cudaError_t launch_gather(const QueryOut& o, const uint64_t* id_offsets, uint64_t n, uint32_t* ids,
                           DevStatus* st, cudaStream_t s, const uint64_t* n_dev, uint64_t ids_cap) {
     if (n == 0) return cudaSuccess;
-    // one resident wave of warps serving the work queue
+    // one resident wave of blocks serving the work queue, or a block a part
     static int wave[64] = {0};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -678,9 +774,12 @@ cudaError_t launch_gather(const QueryOut& o, const uint64_t* id_offsets, uint64_
         if (e != cudaSuccess) return e;
         wave[dev] = sms * (per_sm > 0 ? per_sm : 1);
     }
-    const int most = dev < 64 ? wave[dev] : 152 * 4;
-    int blocks = grid_for(n * 32, GA_THREADS, most);
-    k_gather<<<blocks, GA_THREADS, 0, s>>>(o, id_offsets, n, ids, st, n_dev, ids_cap);
+    // (no more warps than the smallest parts of n answers)
+    const uint64_t most = dev < 64 ? wave[dev] : 152 * 4;
+    const uint64_t parts = o.bits_words ? (o.bits_words + GA_PART_LEAST - 1) / GA_PART_LEAST : 16;
+    const uint64_t want = n >= most * GA_WARPS ? most : (n * parts + GA_WARPS - 1) / GA_WARPS;
+    const uint64_t blocks = std::min(most, want);
+    k_gather<<<(unsigned)blocks, GA_THREADS, 0, s>>>(o, id_offsets, n, ids, st, n_dev, ids_cap);
     return cudaGetLastError();
 }
 
