@@ -32,6 +32,10 @@ cudaError_t launch_probe(const IndexView& ix, const HashParams& hp, const BatchV
                          const QueryTuning& t, DevStatus* st, cudaStream_t s, int* n_launched) {
     *n_launched = 0;
     if (b.n == 0 && !b.desc) return cudaSuccess;
+    if (t.wide) {
+        *n_launched = 1;
+        return launch_query_wide(ix, hp, b, o, t.blocks, st, s);
+    }
     // Which instances the batch needs: known here for a batch sized on the
     // host.  For one sized on the device every instance that can be the
     // batch's is launched, and the others return at once; sequences are not

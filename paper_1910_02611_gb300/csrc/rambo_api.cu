@@ -610,11 +610,17 @@ int resolve_tuning(rambo* h, uint64_t n, int& use_bitmap, QueryTuning& t) {
         use_bitmap = 0;
         t.wide = 1;
         t.set_stage = 1;
-        const int per_sm = query_wide_blocks_per_sm(h->R, h->S);
-        if (per_sm < 1) return RAMBO_EINVAL;
-        uint64_t blocks = (uint64_t)per_sm * h->num_sms;
+        if (!h->tuned_known) {
+            h->tuned = rambo::Tuned{};
+            h->tuned.per_sm = query_wide_blocks_per_sm(h->R, h->S, h->eta);
+            h->tuned.set = set_launch_shape(h->view(), h->num_sms);
+            h->tuned_known = true;
+        }
+        if (h->tuned.per_sm < 1) return RAMBO_EINVAL;
+        uint64_t blocks = (uint64_t)h->tuned.per_sm * h->num_sms;
         if (blocks > n) blocks = n;
         t.blocks = (int)(blocks < 1 ? 1 : blocks);
+        if (h->cfg.set_stage == 0 && h->cfg.answer_staging == 0) t.set = h->tuned.set;
         t.warps_per_block = QW_THREADS / 32;
         t.batch = 1;
         return RAMBO_OK;

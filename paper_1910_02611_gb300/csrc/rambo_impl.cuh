@@ -335,6 +335,8 @@ inline void set_staging(QueryOut& o, uint64_t K, uint32_t staging) {
 // The set kernel's launch (k_query_set.cu).
 struct SetLaunch {
     int qw;        // words of queries per cell (32 * qw queries at a time); 0 = this index is not served
+                   // (wide layouts: tables a pass)
+    bool wide;
     size_t smem;
     int blocks;    // one resident wave
 };
@@ -442,7 +444,7 @@ cudaError_t launch_set(const SetLaunch& sl, const IndexView& ix, const BatchView
 // k_query_wide.cu: block-per-query kernel for wide rows or many tables
 constexpr int QW_THREADS = 256;
 size_t query_wide_smem_bytes(uint32_t R, uint32_t S);
-int query_wide_blocks_per_sm(uint32_t R, uint32_t S);
+int query_wide_blocks_per_sm(uint32_t R, uint32_t S, uint32_t eta);
 cudaError_t launch_query_wide(const IndexView& ix, const HashParams& hp, const BatchView& b, const QueryOut& o,
                               int blocks, DevStatus* st, cudaStream_t s);
 cudaError_t load_query_wide_kernel();
