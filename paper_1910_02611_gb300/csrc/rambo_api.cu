@@ -407,6 +407,7 @@ int insert_bucketed(rambo* h, const BatchView& b, cudaStream_t s) {
     // (48 MiB windows measured faster than 32 MiB ones of a power of two of
     // rows: genome 360 vs 485 ms, uneven 730 vs 866 ms)
     uint64_t rows_per_win = BUCKET_WIN_BYTES / ((uint64_t)h->S * 4);
+    if (rows_per_win >= 8192) rows_per_win &= ~4095ull;  // (the scatter's window quotient is then one multiplication)
     if (rows_per_win < 1) rows_per_win = 1;
     if (rows_per_win > rows_total) rows_per_win = rows_total;
     const uint64_t n_win64 = (rows_total + rows_per_win - 1) / rows_per_win;
@@ -445,7 +446,7 @@ int insert_bucketed(rambo* h, const BatchView& b, cudaStream_t s) {
         }
         for (uint32_t w = 0; w < n_win; ++w)
             CK(launch_bucket_apply(h->rows, (uint64_t)w * rows_per_win * h->S, h->brec.p, h->bfill.p, w, cap,
-                                   h->num_sms, s));
+                                   !b.seq, h->num_sms, s));
     }
     return RAMBO_OK;
 }

@@ -413,7 +413,7 @@ cudaError_t launch_bucket_scatter(const IndexView& ix, const HashParams& hp, con
                                   unsigned long long* fill, unsigned long long* overflow, const DevStatus* st,
                                   int num_sms, cudaStream_t s);
 cudaError_t launch_bucket_apply(uint32_t* rows, uint64_t win_word0, const uint32_t* rec,
-                                const unsigned long long* fill, uint32_t win, uint64_t cap, int num_sms,
+                                const unsigned long long* fill, uint32_t win, uint64_t cap, bool repeats, int num_sms,
                                 cudaStream_t s);
 
 // k_query*.cu
