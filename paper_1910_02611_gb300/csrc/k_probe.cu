@@ -38,11 +38,12 @@ cudaError_t launch_probe(const IndexView& ix, const HashParams& hp, const BatchV
     }
     // Which instances the batch needs: known here for a batch sized on the
     // host.  For one sized on the device every instance that can be the
-    // batch's is launched, and the others return at once; sequences are not
-    // worth the third one (they rarely have eight k-mers).
+    // batch's is launched, and the others return at once (a plan's sequences
+    // are not worth the third one: they rarely have just eight k-mers).
     const int group = t.probe_blocks_group > 0 ? t.group : 1;
-    bool run[3] = {true, t.probe_blocks_group > 0, b.desc ? !b.seq && group <= 1 && b.n >= PB_MANY : false};
-    if (!b.desc) {
+    bool run[3] = {true, t.probe_blocks_group > 0, !(b.desc && b.seq) && group <= 1 && b.n >= PB_MANY};
+    if (b.ends && qk_group_size(b.n, group, (unsigned)t.probe_warps, t.probe_group_warps, 1) == 1) run[PB_GROUP] = false;
+    if (!b.desc && !b.ends) {
         unsigned P;
         const int mode = probe_mode(b, group, (unsigned)t.probe_warps, t.probe_group_warps, 1, P);
         for (int m = 0; m < 3; ++m) run[m] = m == mode;

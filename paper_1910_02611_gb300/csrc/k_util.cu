@@ -21,6 +21,7 @@ __global__ void k_status_reset(DevStatus* st) {
     st->err = NO_ERR;
     st->bad_pos = NO_ERR;
     st->ticket = 0;
+    st->total = 0;
     st->gather_ticket = 0;
     st->n_handed = 0;
     st->set_done = 0;
@@ -112,6 +113,10 @@ cudaError_t launch_or_words(uint32_t* dst, const uint32_t* src, uint64_t n, cuda
 __device__ __forceinline__ void validate_items(const BatchView& b, uint64_t min_len, unsigned short_prio, uint64_t K,
                                                DevStatus* st, uint64_t t0, uint64_t stride) {
     if (b.desc && t0 == 0 && (b.offsets[0] != 0 || b.offsets[b.n] != b.total)) record_error(st, 0, PRIO_EINVAL);
+    if (b.ends && t0 == 0) {
+        if (b.offsets[b.n] < b.offsets[0]) record_error(st, 0, PRIO_EINVAL);
+        st->total = b.total;
+    }
     for (uint64_t t = t0; t < b.n; t += stride) {
         if (b.set_ids && b.set_ids[t] >= K) {
             record_error(st, t, PRIO_ERANGE);
@@ -248,7 +253,13 @@ __global__ void k_intake(BatchView b, uint64_t min_len, unsigned short_prio, uin
     bv_resolve(b);
     const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x, stride = (uint64_t)gridDim.x * blockDim.x;
     validate_items(b, min_len, short_prio, K, st, t0, stride);
-    if (bases) pack_words(bases, b.total, packed, b.desc ? b.total / 32 + 2 : n_words, st, nmask, t0, stride);
+    if (!bases) return;
+    const uint64_t words = b.total / 32 + 2;
+    if (b.ends && words > n_words) {  // (n_words: the packed buffer's capacity)
+        if (t0 == 0) record_error(st, 0, PRIO_GROW);
+        return;
+    }
+    pack_words(bases + (b.ends ? b.off0 : 0), b.total, packed, b.desc || b.ends ? words : n_words, st, nmask, t0, stride);
 }
 
 cudaError_t launch_intake(const BatchView& b, uint64_t min_len, uint64_t K, const uint8_t* bases, uint64_t* packed,
@@ -256,7 +267,12 @@ cudaError_t launch_intake(const BatchView& b, uint64_t min_len, uint64_t K, cons
     if (b.n == 0 && !b.desc) return cudaSuccess;
     const unsigned prio = b.seq ? PRIO_EBADSEQ : PRIO_EINVAL;
     const uint64_t work = b.n > n_words ? b.n : n_words;  // capacities for a descriptor batch
-    k_intake<<<grid_for(work, 256, 1 << 16), 256, 0, s>>>(b, min_len, prio, K, bases, packed, n_words, nmask, st);
+    // a batch sized on the device: for eight words a query, 64 blocks at least
+    // (one long sequence) and one resident wave at most
+    const int blocks = !b.ends ? grid_for(work, 256, 1 << 16)
+                       : bases ? std::max(64, grid_for(b.n * 8, 256, 152 * 8))
+                               : grid_for(b.n, 256, 152 * 8);
+    k_intake<<<blocks, 256, 0, s>>>(b, min_len, prio, K, bases, packed, n_words, nmask, st);
     return cudaGetLastError();
 }
 

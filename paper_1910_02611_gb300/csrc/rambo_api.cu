@@ -101,6 +101,13 @@ uint32_t stride_for(uint32_t W) {
     return (W + 3) / 4 * 4;
 }
 
+// the handle's small block: status, then a small query's inputs
+constexpr size_t BLK_STATUS = 256, BLK_INPUT = 64 * 1024;
+static_assert(sizeof(DevStatus) <= BLK_STATUS, "the status block fits its slot");
+// answers in host memory: up to this many IDs and offsets are copied along
+// with the status, before their number is known
+constexpr uint64_t EARLY_IDS = 16384;
+
 // default build window: a slice of the index that stays resident in L2
 constexpr uint64_t BUILD_TILE_BYTES = 128ull << 20;  // measured fastest on GB300 (L2 126 MB)
 
@@ -121,9 +128,13 @@ struct rambo {
     uint32_t* mem_ids = nullptr;
     uint4* mem_phi = nullptr;
     uint32_t* mem_bits = nullptr;
-    DevStatus* st = nullptr;
+    DevStatus* st = nullptr;    // at blk
     DevStatus* h_st = nullptr;  // pinned
-    DevStatus* h_reset = nullptr;  // pinned: a clean status block, copied in before each query
+    // One device block and its pinned mirror: the status block, then room for
+    // a small query's inputs, so that one copy brings both.  The mirror's
+    // status is always the clean one.
+    uint8_t* blk = nullptr;
+    uint8_t* h_blk = nullptr;
     uint64_t* h_small = nullptr;  // pinned, 8 words
     // scratch
     DBuf<uint8_t> in_data;
@@ -144,6 +155,7 @@ struct rambo {
     uint64_t build_tile_bytes = BUILD_TILE_BYTES;
     int build_mode = 0;
     rambo_query_stats_t last{};
+    bool times_due = false;  // last's times are still in the events
     uint64_t launches = 0;
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};  // call start, query start/end, call end
     uint64_t last_err_item = 0;
@@ -197,9 +209,9 @@ void free_handle(rambo* h) {
     if (h->mem_ids) cudaFree(h->mem_ids);
     if (h->mem_phi) cudaFree(h->mem_phi);
     if (h->mem_bits) cudaFree(h->mem_bits);
-    if (h->st) cudaFree(h->st);
+    if (h->blk) cudaFree(h->blk);
     if (h->h_st) cudaFreeHost(h->h_st);
-    if (h->h_reset) cudaFreeHost(h->h_reset);
+    if (h->h_blk) cudaFreeHost(h->h_blk);
     if (h->h_small) cudaFreeHost(h->h_small);
     for (auto& e : h->ev)
         if (e) cudaEventDestroy(e);
@@ -696,19 +708,21 @@ bool probe_room(rambo* h, uint64_t n, const QueryTuning& t) {
 // else the query kernel alone), and the counts scanned into CSR offsets.
 int enqueue_answers(rambo* h, const BatchView& b, const QueryOut& o, const QueryTuning& t, int use_bitmap,
                     uint64_t* d_off, const uint64_t* base_dev, cudaEvent_t staged, cudaStream_t s) {
+    unsigned long long* total_out = &h->st->spare[1];
     int nl = 0, n_scan = 0;
     bool scanned = false;
     if (o.dmask) {
         CK(launch_probe(h->view(), h->hp, b, o, t, h->st, s, &nl));
         scanned = b.n <= SET_SCAN_MAX;
-        CK(launch_set(t.set, h->view(), b, o, scanned, d_off, base_dev, nullptr, h->st, s));
+        CK(launch_set(t.set, h->view(), b, o, scanned, d_off, base_dev, total_out, h->st, s));
         ++nl;
     } else {
         CK(launch_query(h->view(), h->hp, b, o, t, use_bitmap, h->st, s, &nl));
     }
     if (staged) CK(cudaEventRecord(staged, s));
     if (!scanned)
-        CK(launch_scan_counts(o.qcount, b.n, d_off, h->scan_tmp.p, h->scan_tmp.cap, s, nullptr, &n_scan, base_dev));
+        CK(launch_scan_counts(o.qcount, b.n, d_off, h->scan_tmp.p, h->scan_tmp.cap, s, nullptr, &n_scan, base_dev,
+                              total_out));
     h->launches += (uint64_t)(nl + n_scan);
     return RAMBO_OK;
 }
@@ -717,14 +731,15 @@ int enqueue_answers(rambo* h, const BatchView& b, const QueryOut& o, const Query
 // from the pinned template -- a copy, not a kernel -- then the intake:
 // validation and 2-bit packing in one launch (the query kernel looks up the
 // item of an unresolved base, if packing met one).  Sets the batch's packed,
-// mask or key pointers.
-int enqueue_intake(rambo* h, BatchView& b, const void* d_data, int seq, uint32_t k, cudaStream_t s) {
-    CK(cudaMemcpyAsync(h->st, h->h_reset, sizeof(DevStatus), cudaMemcpyHostToDevice, s));
+// mask or key pointers.  `fresh`: the inputs' copy brought a clean status.
+int enqueue_intake(rambo* h, BatchView& b, const void* d_data, int seq, uint32_t k, bool fresh, cudaStream_t s) {
+    if (!fresh) CK(cudaMemcpyAsync(h->st, h->h_blk, sizeof(DevStatus), cudaMemcpyHostToDevice, s));
     const uint8_t* bases = nullptr;
     uint64_t n_words = 0;
     b.nmask = nullptr;
     if (seq) {
-        n_words = b.total / 32 + 2;  // one spare word for windows crossing the last word
+        // (sized on the device: as many words as there are; the intake says so when they are too few)
+        n_words = b.ends ? h->packed.cap : b.total / 32 + 2;  // one spare word for windows crossing the last word
         RK(h->packed.ensure(n_words));
         b.packed = h->packed.p;
         if (b.skipn) {
@@ -782,7 +797,7 @@ int run_query_pipelined(rambo* h, BatchView b, const void* d_data, int seq, uint
     const bool probe = probe_room(h, n / (uint64_t)C + 1, t0);
 
     CK(cudaEventRecord(h->ev[0], s));
-    RK(enqueue_intake(h, b, d_data, seq, k, s));
+    RK(enqueue_intake(h, b, d_data, seq, k, false, s));
     // the item holding an unresolved base, looked up over the whole batch
     // (the chunks' query kernels see only their slice)
     if (seq) {
@@ -875,6 +890,7 @@ int run_query(rambo* h, int seq, const void* data, const uint64_t* offsets, uint
     k = kk;
     CK(cudaSetDevice(h->device));
     h->last = rambo_query_stats_t{};
+    h->times_due = false;
     h->launches = 0;
     if (n == 0) {
         if (d.arena) {
@@ -905,7 +921,10 @@ int run_query(rambo* h, int seq, const void* data, const uint64_t* offsets, uint
     b.canon = canon;
     b.skipn = skipn;
     const void* d_data = nullptr;
-    RK(stage_batch(h, data, seq ? 1 : 8, offsets, nullptr, n, on_device, s, b, &d_data));
+    const size_t elem = seq ? 1 : 8;
+    bool fresh = false;  // the status block is clean already
+    const bool piped = !on_device && d.arena && n >= PIPE_MIN_QUERIES && !h->cfg.cluster && !h->cfg.l2_fetch_bytes &&
+                       h->cfg.host_chunks != 1;
     int use_bitmap = 0;
     QueryTuning t{};
     RK(resolve_tuning(h, n, use_bitmap, t));
@@ -914,8 +933,29 @@ int run_query(rambo* h, int seq, const void* data, const uint64_t* offsets, uint
     RK(h->scan_tmp.ensure(scan_tmp_words(n)));
     const bool probe = probe_room(h, n, t);
     if (!probe && h->stage.cap < (1u << 20)) RK(h->stage.ensure(1u << 20));
-    if (!on_device && d.arena && n >= PIPE_MIN_QUERIES && !h->cfg.cluster && !h->cfg.l2_fetch_bytes &&
-        h->cfg.host_chunks != 1) {
+    if (on_device && !h->cfg.cluster && (!seq || h->packed.p)) {
+        // the kernels read where the batch starts and ends; nothing waits for it here
+        b.n = n;
+        b.offsets = offsets;
+        b.ends = 1;
+        d_data = data;
+    } else if (!on_device && offsets[n] >= offsets[0] && n < BLK_INPUT / 16 &&
+               (offsets[n] - offsets[0]) * elem <= BLK_INPUT - 16 - 8 * (n + 1)) {
+        // small host inputs and the clean status block in one copy
+        b.n = n;
+        b.off0 = offsets[0];
+        b.total = offsets[n] - offsets[0];
+        const size_t off_bytes = ((n + 1) * 8 + 15) & ~(size_t)15;
+        std::memcpy(h->h_blk + BLK_STATUS, offsets, (n + 1) * 8);
+        std::memcpy(h->h_blk + BLK_STATUS + off_bytes, static_cast<const uint8_t*>(data) + b.off0 * elem, b.total * elem);
+        CK(cudaMemcpyAsync(h->blk, h->h_blk, BLK_STATUS + off_bytes + b.total * elem, cudaMemcpyHostToDevice, s));
+        b.offsets = reinterpret_cast<const uint64_t*>(h->blk + BLK_STATUS);
+        d_data = h->blk + BLK_STATUS + off_bytes;
+        fresh = true;
+    } else {
+        RK(stage_batch(h, data, elem, offsets, nullptr, n, on_device, s, b, &d_data));
+    }
+    if (piped) {
         const int rc = run_query_pipelined(h, b, d_data, seq, k, n, s, d);
         if (rc != PIPE_FALLBACK) return rc;
         h->launches = 0;
@@ -928,9 +968,21 @@ int run_query(rambo* h, int seq, const void* data, const uint64_t* offsets, uint
         RK(h->id_off.ensure(n + 1));
         d_off = h->id_off.p;
     }
-    for (int attempt = 0; attempt < 2; ++attempt) {
+    // the IDs go straight to the caller's device buffer, else to the handle's,
+    // as large as it is already (the gather leaves answers that do not fit)
+    const bool to_caller = !d.arena && on_device;
+    uint64_t early = 0;  // IDs copied to pinned memory before their number is known
+    if (!on_device) {
+        RK(h->h_id_off.ensure(n + 1));
+        if (n < EARLY_IDS) early = std::min(EARLY_IDS, (uint64_t)h->ids.cap);
+        if (early) RK(h->h_ids.ensure(early));
+    }
+    uint64_t total_ids = 0;
+    QueryOut o{};
+    for (int attempt = 0; attempt < 2;) {
         CK(cudaEventRecord(h->ev[0], s));
-        RK(enqueue_intake(h, b, d_data, seq, k, s));
+        RK(enqueue_intake(h, b, d_data, seq, k, fresh, s));
+        fresh = false;
         b.perm = nullptr;
         if (h->cfg.cluster) {
             RK(h->ckeys.ensure(n));
@@ -943,7 +995,7 @@ int run_query(rambo* h, int seq, const void* data, const uint64_t* offsets, uint
             b.perm = h->perm.p;
             h->launches += 5;
         }
-        QueryOut o{h->stage.p, h->stage.cap, h->qstart.p, h->qcount.p};
+        o = QueryOut{h->stage.p, h->stage.cap, h->qstart.p, h->qcount.p};
         set_staging(o, h->K, h->cfg.answer_staging);
         if (probe) o.dmask = h->dmask.p, o.dq = h->dq.p, o.dlong = h->dq.p + h->dq.cap / 2;
         size_t l2_prev = 0;
@@ -954,15 +1006,28 @@ int run_query(rambo* h, int seq, const void* data, const uint64_t* offsets, uint
         CK(cudaEventRecord(h->ev[1], s));
         RK(enqueue_answers(h, b, o, t, use_bitmap, d_off, nullptr, h->ev[2], s));
         if (h->cfg.l2_fetch_bytes) CK(cudaDeviceSetLimit(cudaLimitMaxL2FetchGranularity, l2_prev));
+        CK(launch_gather(o, d_off, n, to_caller ? d.ids : h->ids.p, h->st, s, nullptr, to_caller ? d.ids_cap : h->ids.cap));
+        CK(cudaEventRecord(h->ev[3], s));
+        h->launches += 1;
         CK(cudaMemcpyAsync(h->h_st, h->st, sizeof(DevStatus), cudaMemcpyDeviceToHost, s));
-        CK(cudaMemcpyAsync(h->h_small, d_off + n, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+        if (early) {
+            CK(cudaMemcpyAsync(h->h_id_off.p, d_off, (n + 1) * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+            CK(cudaMemcpyAsync(h->h_ids.p, h->ids.p, early * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        }
         CK(cudaStreamSynchronize(s));
+        if (h->h_st->err != NO_ERR && (h->h_st->err & 0xff) == PRIO_GROW) {
+            // a batch sized on the device that the packed buffer does not hold: grow it and run again
+            RK(h->packed.ensure(h->h_st->total / 32 + 2));
+            h->launches = 0;
+            continue;
+        }
         RK(decode_err(h, h->h_st->err));
+        total_ids = h->h_st->spare[1];
         if (h->h_st->cursor <= h->stage.cap) break;
-        if (attempt == 1) return RAMBO_ECUDA;  // the second run needs exactly the first's count
+        if (++attempt == 2) return RAMBO_ECUDA;  // the second run needs exactly the first's count
         RK(h->stage.ensure(h->h_st->cursor + (h->h_st->cursor >> 3)));
     }
-    const uint64_t total_ids = h->h_small[0];
+    if (b.ends) b.total = h->h_st->total;
     h->last.n_queries = n;
     h->last.keys_submitted = seq ? (b.total - n * (uint64_t)(k - 1)) : b.total;
     h->last.keys_probed = h->h_st->keys_probed;
@@ -970,59 +1035,61 @@ int run_query(rambo* h, int seq, const void* data, const uint64_t* offsets, uint
     h->last.n_results = total_ids;
     for (int i = 0; i < 4; ++i) h->last.stage_queries[i] = h->h_st->stage_count[i];
     h->last.staged_words = h->h_st->cursor;
-    CK(cudaEventElapsedTime(&h->last.query_kernel_ms, h->ev[1], h->ev[2]));
+    h->times_due = true;
     if (d.needed) *d.needed = total_ids;
     if (!d.arena && total_ids > d.ids_cap) return RAMBO_ENOSPC;
-    QueryOut o{h->stage.p, h->stage.cap, h->qstart.p, h->qcount.p};
-    set_staging(o, h->K, h->cfg.answer_staging);
-    if (on_device) {
-        uint32_t* d_ids;
-        if (!d.arena) {
-            d_ids = d.ids;
-        } else {
-            RK(h->ids.ensure(total_ids + 1));
-            d_ids = h->ids.p;
-        }
-        CK(launch_gather(o, d_off, n, d_ids, h->st, s));
+    if (!to_caller && total_ids > h->ids.cap) {
+        // the handle's buffer was too small: grow it and gather again
+        RK(h->ids.ensure(total_ids + 1));
+        CK(launch_gather(o, d_off, n, h->ids.p, h->st, s));
         CK(cudaEventRecord(h->ev[3], s));
         h->launches += 1;
-        h->last.kernel_launches = h->launches;
-        CK(cudaStreamSynchronize(s));
-        CK(cudaEventElapsedTime(&h->last.device_ms, h->ev[0], h->ev[3]));
+        early = 0;
+        if (on_device) CK(cudaStreamSynchronize(s));
+    }
+    h->last.kernel_launches = h->launches;
+    if (on_device) {
         if (d.arena) {
-            *d.out_ids = d_ids;
+            RK(h->ids.ensure(total_ids + 1));
+            *d.out_ids = h->ids.p;
             *d.out_off = d_off;
         }
         return RAMBO_OK;
     }
-    uint32_t* hid;
-    uint64_t* hoff;
+    uint32_t* hid = d.ids;
+    uint64_t* hoff = d.id_offsets;
     if (d.arena) {
-        RK(h->h_ids.ensure(total_ids + 1));
-        RK(h->h_id_off.ensure(n + 1));
+        if (!early || total_ids > early) RK(h->h_ids.ensure(total_ids + 1));
         hid = h->h_ids.p;
         hoff = h->h_id_off.p;
-    } else {
-        hid = d.ids;
-        hoff = d.id_offsets;
     }
-    // (Gathering large answers straight into pinned host memory over
-    // NVLink-C2C measured slower than gathering on the device and copying:
-    // 1.9e6 against 2.15e6 keys/s end to end on the document workload.)
-    RK(h->ids.ensure(total_ids + 1));
-    uint32_t* d_ids = h->ids.p;
-    CK(launch_gather(o, d_off, n, d_ids, h->st, s));
-    CK(cudaEventRecord(h->ev[3], s));
-    h->launches += 1;
-    h->last.kernel_launches = h->launches;
-    CK(cudaMemcpyAsync(hoff, d_off, (n + 1) * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-    if (total_ids) CK(cudaMemcpyAsync(hid, d_ids, total_ids * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    CK(cudaEventElapsedTime(&h->last.device_ms, h->ev[0], h->ev[3]));
+    if (early && total_ids <= early) {
+        // everything is in pinned memory
+        if (!d.arena) {
+            std::memcpy(hoff, h->h_id_off.p, (n + 1) * sizeof(uint64_t));
+            std::memcpy(hid, h->h_ids.p, total_ids * sizeof(uint32_t));
+        }
+    } else {
+        // (Gathering large answers straight into pinned host memory over
+        // NVLink-C2C measured slower than gathering on the device and copying:
+        // 1.9e6 against 2.15e6 keys/s end to end on the document workload.)
+        CK(cudaMemcpyAsync(hoff, d_off, (n + 1) * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+        if (total_ids) CK(cudaMemcpyAsync(hid, h->ids.p, total_ids * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+    }
     if (d.arena) {
         *d.out_ids = hid;
         *d.out_off = hoff;
     }
+    return RAMBO_OK;
+}
+
+// The times of the last query call, read from its events when they are asked for.
+int settle_times(rambo* h) {
+    if (!h->times_due) return RAMBO_OK;
+    h->times_due = false;
+    CK(cudaEventElapsedTime(&h->last.query_kernel_ms, h->ev[1], h->ev[2]));
+    CK(cudaEventElapsedTime(&h->last.device_ms, h->ev[0], h->ev[3]));
     return RAMBO_OK;
 }
 
@@ -1115,12 +1182,16 @@ static int create_impl(uint64_t K, uint32_t B_local, uint32_t n_nodes, uint32_t 
     if (cudaMalloc(&h->rows, h->index_words() * 4) != cudaSuccess) return fail(RAMBO_ENOMEM);
     if (cudaMalloc(&h->phi, K * phi_stride_for(R) * sizeof(uint16_t)) != cudaSuccess) return fail(RAMBO_ENOMEM);
     if (cudaMalloc(&h->reg, ((K + 31) / 32) * 4) != cudaSuccess) return fail(RAMBO_ENOMEM);
-    if (cudaMalloc(&h->st, sizeof(DevStatus)) != cudaSuccess) return fail(RAMBO_ENOMEM);
+    if (cudaMalloc(&h->blk, BLK_STATUS + BLK_INPUT) != cudaSuccess) return fail(RAMBO_ENOMEM);
+    h->st = reinterpret_cast<DevStatus*>(h->blk);
     if (cudaMallocHost(&h->h_st, sizeof(DevStatus)) != cudaSuccess) return fail(RAMBO_ENOMEM);
-    if (cudaMallocHost(&h->h_reset, sizeof(DevStatus)) != cudaSuccess) return fail(RAMBO_ENOMEM);
-    *h->h_reset = DevStatus{};
-    h->h_reset->err = NO_ERR;
-    h->h_reset->bad_pos = NO_ERR;
+    if (cudaMallocHost(&h->h_blk, BLK_STATUS + BLK_INPUT) != cudaSuccess) return fail(RAMBO_ENOMEM);
+    {
+        DevStatus clean{};
+        clean.err = NO_ERR;
+        clean.bad_pos = NO_ERR;
+        std::memcpy(h->h_blk, &clean, sizeof(clean));
+    }
     if (cudaMallocHost(&h->h_small, 8 * sizeof(uint64_t)) != cudaSuccess) return fail(RAMBO_ENOMEM);
     for (auto& ev : h->ev)
         if (cudaEventCreate(&ev) != cudaSuccess) return fail(RAMBO_ECUDA);
@@ -1402,6 +1473,7 @@ int rambo_cell_popcount(const rambo_t* h, uint64_t* host_out, void* stream) {
 
 int rambo_last_query_stats(const rambo_t* h, rambo_query_stats_t* out) {
     if (!h || !out) return RAMBO_EINVAL;
+    RK(settle_times(const_cast<rambo*>(h)));
     *out = h->last;
     return RAMBO_OK;
 }
@@ -1534,6 +1606,7 @@ int rambo_autotune(rambo_t* h, int kind, const void* data, const uint64_t* offse
                     h->cfg = keep;
                     return rc;
                 }
+                RK(settle_times(h));
                 if (t_min < 0 || h->last.device_ms < t_min) t_min = h->last.device_ms;
             }
             if (win_ms < 0 || t_min < win_ms) {

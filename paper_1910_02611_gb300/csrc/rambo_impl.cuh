@@ -28,6 +28,7 @@ constexpr unsigned long long NO_ERR = ~0ull;
 // Device error word: (index << 8) | priority; the smallest value wins, so the
 // lowest-numbered bad item is reported.  Priorities, lowest first, follow the
 // order in which items are checked: set ID range, offsets, content.
+constexpr unsigned PRIO_GROW = 0;  // (no item's error: the packed buffer is too small for a batch sized on the device)
 constexpr unsigned PRIO_ERANGE = 1;
 constexpr unsigned PRIO_EINVAL = 2;
 constexpr unsigned PRIO_EBADSEQ = 3;
@@ -47,6 +48,7 @@ struct DevStatus {
     unsigned long long rows_read;    // row reads issued
     unsigned long long spare[2];
     unsigned long long stage_count[4];   // surviving queries per set stage (1 dense, 2 sparse, 3 union)
+    unsigned long long total;            // data items of a batch sized on the device
 };
 constexpr size_t QUEUE_BYTES = 6 * sizeof(unsigned long long);  // ticket .. ticket_long
 
@@ -257,10 +259,22 @@ struct BatchView {
     const uint64_t* desc;          // device descriptor {n, total} (offsets[0] = 0) read at
                                    // kernel start instead of n/total/off0; lets one captured
                                    // CUDA graph serve batches of any size up to its capacity
+    int ends;                      // 1: n is known, off0 and total come from the device's own
+                                   // offsets (the host does not wait for them); keys and bases
+                                   // then start at item 0 of the caller's data
 };
 
-// Takes n, total and off0 from the device descriptor when there is one.
+// Takes n, total and off0 from the device descriptor when there is one, or
+// off0 and total from the offsets (none when they end before they start: the
+// validation reports that).
 __device__ __forceinline__ void bv_resolve(BatchView& b) {
+    if (b.ends) {
+        const uint64_t lo = __ldg(b.offsets), hi = __ldg(b.offsets + b.n);
+        b.off0 = lo;
+        b.total = hi < lo ? 0 : hi - lo;
+        if (!b.seq) b.keys += lo;
+        return;
+    }
     if (b.desc) {
         b.n = b.desc[0];
         b.total = b.desc[1];

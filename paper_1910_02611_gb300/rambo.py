@@ -163,7 +163,7 @@ def _stream_handle(stream) -> int | None:
     if stream is None:
         try:
             torch = _torch()
-            if torch.cuda.is_available() and torch.cuda.is_initialized():
+            if torch.cuda.is_initialized():
                 return torch.cuda.current_stream().cuda_stream
         except ImportError:  # pragma: no cover
             pass
@@ -192,6 +192,18 @@ def _device_copy(ptr: int, n: int, dtype: str, copy: bool = True):
         return torch.zeros(0, dtype=tdt, device="cuda")
     t = torch.as_tensor(_CudaArray(ptr, n, "<i4" if dtype == "<u4" else "<i8"), device="cuda")
     return t.clone() if copy else t
+
+
+class _HostArray:
+    """Exposes n values of host memory at ptr through __array_interface__."""
+
+    def __init__(self, ptr: int, n: int, typestr: str):
+        self.__array_interface__ = {"shape": (n,), "typestr": typestr, "data": (ptr, False), "version": 3}
+
+
+def _host_view(ptr: int, n: int, typestr: str) -> np.ndarray:
+    """A numpy view of host memory (ctypes' as_array costs ten times as much)."""
+    return np.asarray(_HostArray(ptr, n, typestr))
 
 
 def _host_arr(x, dtype) -> np.ndarray:
@@ -348,12 +360,12 @@ class Rambo:
             off_t = _device_copy(offo_p.value, n + 1, "<u8", copy)
             total = int(off_t[-1].item())
             return _device_copy(ids_p.value or 0, total, "<u4", copy), off_t
-        offs = np.ctypeslib.as_array(C.cast(offo_p, C.POINTER(_u64)), shape=(n + 1,))
+        offs = _host_view(offo_p.value, n + 1, "<u8")
         offs = offs.copy() if copy else offs
         total = int(offs[-1])
         if total == 0:
             return np.zeros(0, np.uint32), offs
-        ids = np.ctypeslib.as_array(C.cast(ids_p, C.POINTER(_u32)), shape=(total,))
+        ids = _host_view(ids_p.value, total, "<u4")
         return (ids.copy() if copy else ids), offs
 
     def query_into(self, data, offsets, ids_out, id_offsets_out, kind: str = "keys", k: int = 31, stream=None) -> int:
@@ -583,9 +595,8 @@ class Plan:
         if not copy and not to_host:
             return ids_p.value, off_p.value, total
         if to_host:
-            offs = np.ctypeslib.as_array(C.cast(off_p, C.POINTER(_u64)), shape=(n + 1,)).copy()
-            ids = (np.ctypeslib.as_array(C.cast(ids_p, C.POINTER(_u32)), shape=(total,)).copy() if total
-                   else np.zeros(0, np.uint32))
+            offs = _host_view(off_p.value, n + 1, "<u8").copy()
+            ids = _host_view(ids_p.value, total, "<u4").copy() if total else np.zeros(0, np.uint32)
             return ids, offs
         return _device_copy(ids_p.value or 0, total, "<u4"), _device_copy(off_p.value, n + 1, "<u8")
 
