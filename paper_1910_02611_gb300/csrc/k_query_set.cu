@@ -215,11 +215,18 @@ __device__ __forceinline__ void scan_counts_block(const uint32_t* counts, uint64
         const uint64_t i0 = base + (uint64_t)threadIdx.x * PER;
         uint32_t v[PER];
         uint64_t sum = 0;
+        if (i0 + PER <= n && (reinterpret_cast<uintptr_t>(counts) & 15) == 0) {
 #pragma unroll
-        for (int t = 0; t < PER; ++t) {
-            v[t] = i0 + t < n ? __ldcg(counts + i0 + t) : 0u;
-            sum += v[t];
+            for (int t = 0; t < PER; t += 4) {
+                const uint4 x = __ldcg(reinterpret_cast<const uint4*>(counts + i0 + t));
+                v[t] = x.x, v[t + 1] = x.y, v[t + 2] = x.z, v[t + 3] = x.w;
+            }
+        } else {
+#pragma unroll
+            for (int t = 0; t < PER; ++t) v[t] = i0 + t < n ? __ldcg(counts + i0 + t) : 0u;
         }
+#pragma unroll
+        for (int t = 0; t < PER; ++t) sum += v[t];
         uint64_t incl = sum;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
@@ -426,9 +433,13 @@ cudaError_t launch_set(const SetLaunch& sl, const IndexView& ix, const BatchView
                        uint64_t* id_offsets, const uint64_t* base_dev, unsigned long long* total_out, DevStatus* st,
                        cudaStream_t s) {
     if (b.n == 0 && !b.desc) return cudaSuccess;
-    // no more blocks than there can be items (b.n is the capacity of a descriptor batch)
+    // no more blocks than there can be items (b.n is the capacity of a
+    // descriptor batch): each one that has none still ends in a same-address
+    // atomic, and 456 of them for 40 items cost 5 us
     const uint64_t step = (uint64_t)QS_IDS * (sl.wide ? QSW_WARPS : QS_WARPS);
-    const uint64_t most = b.n * ((ix.K + step - 1) / step);
+    const uint64_t per = sl.wide ? 16 : 32 * (uint64_t)sl.qw;
+    const uint64_t narrow = sl.wide ? 1 : b.n > 32 ? 2 : 1;  // groups of 32 up to 64 queries
+    const uint64_t most = std::max((b.n + per - 1) / per, narrow) * ((ix.K + step - 1) / step);
     const unsigned blocks = (unsigned)((uint64_t)sl.blocks < most ? (uint64_t)sl.blocks : most);
     if (sl.wide)
         k_set_wide<<<blocks, QSW_THREADS, sl.smem, s>>>(ix, b, o, sl.qw, scan, id_offsets, base_dev, total_out, st);

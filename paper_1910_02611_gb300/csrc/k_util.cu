@@ -592,7 +592,7 @@ cudaError_t launch_cluster_order(const BatchView& b, uint64_t* keys, uint32_t* h
 constexpr int GA_THREADS = 256;
 constexpr int GA_WARPS = GA_THREADS / 32;
 constexpr int GA_RUN = 1024;                  // IDs of 32 bitmap words
-constexpr uint32_t GA_SHORT = 4096;           // answers of at most this many IDs are not cut
+constexpr uint32_t GA_SHORT = 4096;           // answers of at most this many IDs are not cut where the grid is filled
 constexpr uint32_t GA_PART_WORDS = 2048;     // bitmap words of a part in a batch that fills the grid,
 constexpr uint32_t GA_PART_LEAST = 128;       // and of the smallest part where it does not
 constexpr unsigned GA_TAKE = 8;               // most parts per work-queue ticket
@@ -709,11 +709,14 @@ __device__ __forceinline__ uint32_t ga_count(const uint32_t* __restrict__ src, u
 }
 
 // Parts a long answer is cut into when n queries share a grid of `warps`.
-__device__ __forceinline__ uint32_t ga_parts(uint32_t bits_words, uint64_t n, uint64_t warps) {
+// Sets the longest answer that stays whole: with warps to spare, none (a few
+// IDs spread over 1e5 bits kept one warp for 50 us).
+__device__ __forceinline__ uint32_t ga_parts(uint32_t bits_words, uint64_t n, uint64_t warps, uint32_t& whole) {
     const uint32_t base = bits_words ? (bits_words + GA_PART_WORDS - 1) / GA_PART_WORDS : 4;
     const uint32_t most = bits_words ? (bits_words + GA_PART_LEAST - 1) / GA_PART_LEAST : 16;
     const uint64_t fill = warps / n;  // parts that occupy every warp
     const uint32_t parts = fill < most ? (uint32_t)fill : most;
+    whole = parts > base ? 0 : GA_SHORT;
     return parts > base ? parts : base;
 }
 
@@ -727,7 +730,8 @@ __global__ void __launch_bounds__(GA_THREADS, 6) k_gather(QueryOut o, const uint
     const unsigned lane = threadIdx.x & 31;
     uint32_t* run = s_run[threadIdx.x >> 5];
     const uint64_t warps = (uint64_t)gridDim.x * GA_WARPS;
-    const uint32_t parts = ga_parts(o.bits_words, n, warps);
+    uint32_t whole;
+    const uint32_t parts = ga_parts(o.bits_words, n, warps, whole);
     const uint64_t units = n * parts;
     // answers that are cut into many parts are taken a part at a time, so that
     // a long one's parts go to several warps; the first take needs no ticket
@@ -741,7 +745,7 @@ __global__ void __launch_bounds__(GA_THREADS, 6) k_gather(QueryOut o, const uint
             const uint64_t q = parts == 1 ? mine : mine / parts;
             part_of = (uint32_t)(mine - q * parts);
             c_of = o.qcount[q];
-            if (part_of && c_of <= GA_SHORT) c_of = 0;
+            if (part_of && c_of <= whole) c_of = 0;
             if (c_of) {
                 s_of = o.qstart[q];
                 d_of = id_offsets[q];
@@ -753,14 +757,14 @@ __global__ void __launch_bounds__(GA_THREADS, 6) k_gather(QueryOut o, const uint
             const uint64_t s0 = __shfl_sync(FULL, s_of, l);
             uint32_t* dst = ids + __shfl_sync(FULL, d_of, l);
             if (!(s0 & QSTART_BITMAP)) {
-                const uint32_t p = c > GA_SHORT ? parts : 1;
+                const uint32_t p = c > whole ? parts : 1;
                 const uint32_t lo = (uint32_t)((uint64_t)c * part / p), hi = (uint32_t)((uint64_t)c * (part + 1) / p);
                 ga_copy(o.stage + s0 + lo, hi - lo, dst + lo, lane);
                 continue;
             }
             const uint32_t* src = o.stage + (s0 & ~QSTART_BITMAP);
             uint32_t w_lo = 0, w_hi = o.bits_words;
-            if (parts > 1 && c > GA_SHORT) {
+            if (parts > 1 && c > whole) {
                 const uint32_t groups = (o.bits_words + 31) / 32;
                 w_lo = (uint32_t)((uint64_t)groups * part / parts) * 32;
                 w_hi = min(w_hi, (uint32_t)((uint64_t)groups * (part + 1) / parts) * 32);
