@@ -223,12 +223,13 @@ def _code_only(text: str) -> str:
 
 
 def kernel_source_hash() -> str:
-    """Hash of the query kernel's device code, comments removed: k_query.cuh,
-    its instantiation header, and the device helpers of rambo_impl.cuh (up to
-    the launcher declarations)."""
+    """Hash of the device code of a plan's query kernels (probes and set
+    stage), comments removed: k_probe.cuh and its instantiation header,
+    k_query.cuh (its helpers), k_query_set.cu, and the device helpers of
+    rambo_impl.cuh (up to the launcher declarations)."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1910_02611_gb300", "csrc")
-    for name in ("k_query.cuh", "k_query_inst.cuh"):
+    for name in ("k_probe.cuh", "k_probe_inst.cuh", "k_query.cuh", "k_query_set.cu"):
         with open(os.path.join(csrc, name)) as f:
             h.update(_code_only(f.read()).encode())
     with open(os.path.join(csrc, "rambo_impl.cuh")) as f:
@@ -238,7 +239,7 @@ def kernel_source_hash() -> str:
 
 
 def ncu_traffic(config: str):
-    """Per-launch DRAM bytes of the query kernel from the committed ncu summary,
+    """Per-step DRAM bytes of the query kernels from the committed ncu summary,
     valid only while the kernel source is the one that was profiled."""
     p = os.path.join(ROOT, "profiles", f"query_kernel_{config}_traffic.txt")
     if not os.path.exists(p):
@@ -657,7 +658,7 @@ def run_ours(args):
         "roofline": {
             "bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
             "frac": achieved / peaks["hbm_gbs"], "traffic": ncu_traffic(w.name),
-            "kernel": "k_query", "peak_source": peaks["source"],
+            "kernel": "k_probe + k_set", "peak_source": peaks["source"],
             "bytes_model": f"rows read (device counter) x {sectors_per_row} sector(s) x 32 B + 4 B per staged word "
                            "(an ID of a list-staged answer or a word of a bitmap-staged one; device counter)",
             "staged_words_per_step": staged / args.steps,

@@ -434,7 +434,8 @@ typedef struct rambo_query_stats {
     float query_kernel_ms;
     float device_ms;
     uint64_t stage_queries[4];  /* queries that reached the set stage, by stage used:
-                                 * [0] staged dense (large ID space), [1] dense,
+                                 * [0] staged dense (large ID space), [1] dense
+                                 * (in the query kernel or the set kernel),
                                  * [2] sparse, [3] union */
     uint64_t staged_words;      /* 32-bit words the query kernel wrote to the
                                  * staging arena: ID lists and set bitmaps */
@@ -447,7 +448,10 @@ int rambo_last_query_stats(const rambo_t *h, rambo_query_stats_t *out);
  *   warps_per_block (1, 2, 4 or 8; 0 = automatic: the largest block that
  *   keeps at least 85% of the most warps resident per SM),
  *   blocks_per_sm (0 = as many as fit),
- *   set_stage: 0 = auto, 1 = dense scan of the partition table,
+ *   set_stage: 0 = auto (batches of more than the smallest size: probe and set
+ *              kernels, when row_load and answer_staging are at their
+ *              defaults too and memory holds a bitmap a query),
+ *              1 = dense scan of the partition table,
  *              2 = sparse enumeration of the hit cells' members,
  *              3 = union of the hit cells' member bitmaps (complemented for
  *                  tables with most cells hit), per table, intersected,
@@ -491,7 +495,8 @@ typedef struct rambo_query_config {
                                * piece, copied at the end; at most 8 */
     uint32_t answer_staging;  /* how a query's answer waits in the staging
                                * arena before it is laid out in query order:
-                               * 0 = automatic (as its K-bit set bitmap when it
+                               * 0 = automatic (from the set kernel as its K-bit
+                               * set bitmap; from the query kernel so when it
                                * holds more IDs than the bitmap has 32-bit
                                * words, else as its ID list); 1 = always as
                                * the ID list; f = 2..64: as the bitmap only

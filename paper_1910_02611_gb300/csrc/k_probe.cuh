@@ -3,9 +3,13 @@
 // (k_query_set.cu).  Steps A1-A4 are those of k_query.cuh; a query whose R
 // per-table cell masks all keep a hit cell is handed over as those masks.
 //
-// Without a set stage a warp needs no shared-memory bitmap of the ID space,
-// so the row reads, which are what the kernel waits for, have every warp of
-// the SM in flight (document workload, K = 1e5: 48 warps instead of 16).
+// Without a set stage a warp needs no shared-memory bitmap of the ID space and
+// nothing holds it up between a query's rows and the next query's.  What
+// bounds it: the rate of isolated DRAM accesses for long queries (1e6 uneven
+// sequences, 7.2e8 rows: 15.4 ms with the set stage in the same kernel, 14.15
+// here; 2e5 short reads 4.77 -> 3.96), latency for short ones, which therefore
+// go 32 / G to a warp (1e5 document queries 0.26 ms, 1e4 single k-mers 33 us by
+// warps, 8 by lane groups).
 //
 // Three instances, picked by the batch's mean number of terms and its size
 // (probe_short, qk_group_size); a launch whose instance is not the batch's

@@ -19,7 +19,7 @@
 // stage with the probes before it, against one query per warp in the query
 // kernel: 1e5 conjunctive queries over 1e5 documents (R = 8, B = 320) 11.7 ms
 // -> 0.26 (probes) + 0.89; 1e4 over 5e5 documents (R = 6, B = 1000; no
-// per-warp bitmap there, so the start scanned all IDs twice) 85.4 ms -> 0.03 +
+// per-warp bitmap there, so a warp scans all IDs twice) 85.4 ms -> 0.03 +
 // 0.54; 16 queries over 1e5 documents 202 us -> 28.
 //
 // Groups of 128 queries are the widest whose T leaves two blocks an SM room;
