@@ -287,12 +287,19 @@ cudaError_t launch_pack(const uint8_t* bases, uint64_t total, uint64_t* packed, 
 // Skip-N queries: query t needs k consecutive resolved bases somewhere in
 // [a, e), i.e. a gap of at least k between consecutive unresolved bases (the
 // range ends counting as unresolved).  Visits only the unresolved bits.
-__global__ void k_check_windows(BatchView b, DevStatus* st) {
+// `mask_words` is the room in nmask: a batch sized on the device that needs
+// more was not packed (PRIO_GROW) and runs again.  The error word is no guide
+// here: other blocks of this launch write it, and every query has to be looked
+// at for the lowest-numbered bad one to be reported.
+__global__ void k_check_windows(BatchView b, uint64_t mask_words, DevStatus* st) {
     bv_resolve(b);
+    if (b.total / 32 + 2 > mask_words) return;
     for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < b.n;
          t += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t a = b.offsets[t] - b.off0, e = b.offsets[t + 1] - b.off0;
-        if (e < a + b.k) continue;  // decreasing or too short: reported by the validation
+        // decreasing, outside the batch or too short: reported by the
+        // validation (of this query, or of a later one that comes back)
+        if (a > e || e > b.total || e - a < b.k) continue;
         uint64_t next = a;          // first base after the last unresolved one seen
         bool found = false;
         for (uint64_t w = a >> 5; w <= (e - 1) >> 5 && !found; ++w) {
@@ -313,9 +320,9 @@ __global__ void k_check_windows(BatchView b, DevStatus* st) {
     }
 }
 
-cudaError_t launch_check_windows(const BatchView& b, DevStatus* st, cudaStream_t s) {
+cudaError_t launch_check_windows(const BatchView& b, uint64_t mask_words, DevStatus* st, cudaStream_t s) {
     if (b.n == 0 && !b.desc) return cudaSuccess;
-    k_check_windows<<<grid_for(b.n, 256, 8192), 256, 0, s>>>(b, st);
+    k_check_windows<<<grid_for(b.n, 256, 8192), 256, 0, s>>>(b, mask_words, st);
     return cudaGetLastError();
 }
 

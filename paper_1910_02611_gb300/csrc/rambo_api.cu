@@ -753,7 +753,7 @@ int enqueue_intake(rambo* h, BatchView& b, const void* d_data, int seq, uint32_t
     CK(launch_intake(b, seq ? k : 1, h->K, bases, h->packed.p, n_words, const_cast<uint32_t*>(b.nmask), h->st, s));
     h->launches += 1;
     if (seq && b.skipn) {
-        CK(launch_check_windows(b, h->st, s));
+        CK(launch_check_windows(b, n_words, h->st, s));
         h->launches += 1;
     }
     return RAMBO_OK;

@@ -390,7 +390,8 @@ cudaError_t launch_validate_batch(const BatchView& b, uint64_t min_len, uint64_t
 cudaError_t launch_pack(const uint8_t* bases, uint64_t total, uint64_t* packed, uint64_t n_words,
                         DevStatus* st, cudaStream_t s, const uint64_t* desc = nullptr, uint32_t* nmask = nullptr);
 // skip-N queries: a query with no window free of unresolved bases is EBADSEQ
-cudaError_t launch_check_windows(const BatchView& b, DevStatus* st, cudaStream_t s);
+// (mask_words: the room in b.nmask)
+cudaError_t launch_check_windows(const BatchView& b, uint64_t mask_words, DevStatus* st, cudaStream_t s);
 cudaError_t launch_resolve_bad_base(const BatchView& b, DevStatus* st, cudaStream_t s);
 cudaError_t launch_register(const BatchView& b, uint32_t* reg, DevStatus* st, cudaStream_t s);
 cudaError_t launch_scan_counts(const uint32_t* counts, uint64_t n, uint64_t* offsets,

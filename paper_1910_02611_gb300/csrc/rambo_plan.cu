@@ -157,7 +157,7 @@ int plan_capture(rambo_plan* p, bool timed) {
         e = launch_intake(b, p->kind ? p->k : 1, ix.K, p->kind == 1 ? p->d_data : nullptr, p->d_packed,
                           p->kind == 1 ? p->max_items / 32 + 2 : 0, p->d_nmask, p->st, s),
         ++n_launch;
-    if (e == cudaSuccess && p->kind == 1 && p->skipn) e = launch_check_windows(b, p->st, s), ++n_launch;
+    if (e == cudaSuccess && p->kind == 1 && p->skipn) e = launch_check_windows(b, p->max_items / 32 + 2, p->st, s), ++n_launch;
     QueryOut o{p->stage, p->stage_words, p->qstart, p->qcount};
     set_staging(o, ix.K, p->staging);
     if (p->probe) o.dmask = p->dmask, o.dq = p->dq, o.dlong = p->dq + p->max_q;
