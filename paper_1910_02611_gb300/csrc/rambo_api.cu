@@ -971,6 +971,7 @@ int run_query(rambo* h, int seq, const void* data, const uint64_t* offsets, uint
     // the IDs go straight to the caller's device buffer, else to the handle's,
     // as large as it is already (the gather leaves answers that do not fit)
     const bool to_caller = !d.arena && on_device;
+    if (!to_caller) RK(h->ids.ensure(1));
     uint64_t early = 0;  // IDs copied to pinned memory before their number is known
     if (!on_device) {
         RK(h->h_id_off.ensure(n + 1));
@@ -1050,8 +1051,7 @@ int run_query(rambo* h, int seq, const void* data, const uint64_t* offsets, uint
     h->last.kernel_launches = h->launches;
     if (on_device) {
         if (d.arena) {
-            RK(h->ids.ensure(total_ids + 1));
-            *d.out_ids = h->ids.p;
+            *d.out_ids = h->ids.p;  // (holds the answers: growing it here would lose them)
             *d.out_off = d_off;
         }
         return RAMBO_OK;
