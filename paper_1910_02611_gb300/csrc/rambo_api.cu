@@ -686,22 +686,30 @@ int resolve_tuning(rambo* h, uint64_t n, int& use_bitmap, QueryTuning& t) {
 constexpr uint64_t PROBE_LEAST_WORDS = 1024;
 
 // Room for an n-query batch on the probe path: a bitmap a query in the
-// staging arena (grown by at most a quarter of the free memory), and masks
-// and indexes of the queries handed over.  False (the query kernel then
-// answers the batch alone) for the smallest batches, when the tuning asks for
-// a set stage or staging form of the query kernel, or when memory is short.
+// staging arena, and masks and indexes of the queries handed over (masks of
+// wide layouts are hundreds of times their bitmaps).  What has to grow takes
+// at most a quarter of the free memory.  False (the query kernel then answers
+// the batch alone) for the smallest batches, when the tuning asks for a set
+// stage or staging form of the query kernel, or when memory is short.
 bool probe_room(rambo* h, uint64_t n, const QueryTuning& t) {
     if (!t.set.qw || n > 0xffffffffull || n * ((h->K + 31) / 32) <= PROBE_LEAST_WORDS) return false;
-    const uint64_t pitch = set_pitch(h->K);
-    if (h->stage.cap / pitch < n) {
-        size_t free_b = 0, total_b = 0;
-        if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || (uint64_t)free_b / 16 / pitch < n) {
-            cudaGetLastError();
-            return false;
-        }
-        if (h->stage.ensure(n * pitch) != RAMBO_OK) return false;
+    const struct {
+        DBuf<uint32_t>& buf;
+        uint64_t words;
+    } want[] = {{h->stage, n * set_pitch(h->K)}, {h->dmask, n * h->R * h->S}, {h->dq, 2 * n}};
+    uint64_t grow = 0;
+    for (const auto& w : want)
+        if (w.buf.cap < w.words) grow += w.words + w.words / 8;
+    if (!grow) return true;
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
     }
-    return h->dmask.ensure(n * h->R * h->S) == RAMBO_OK && h->dq.ensure(2 * n) == RAMBO_OK;
+    if (grow > (uint64_t)free_b / 16) return false;
+    for (const auto& w : want)
+        if (w.buf.ensure(w.words) != RAMBO_OK) return false;
+    return true;
 }
 
 // The queries' answers staged and counted (o.dmask set: probe and set kernel,
@@ -931,8 +939,6 @@ int run_query(rambo* h, int seq, const void* data, const uint64_t* offsets, uint
     RK(h->qcount.ensure(n));
     RK(h->qstart.ensure(n));
     RK(h->scan_tmp.ensure(scan_tmp_words(n)));
-    const bool probe = probe_room(h, n, t);
-    if (!probe && h->stage.cap < (1u << 20)) RK(h->stage.ensure(1u << 20));
     if (on_device && !h->cfg.cluster && (!seq || h->packed.p)) {
         // the kernels read where the batch starts and ends; nothing waits for it here
         b.n = n;
@@ -960,6 +966,9 @@ int run_query(rambo* h, int seq, const void* data, const uint64_t* offsets, uint
         if (rc != PIPE_FALLBACK) return rc;
         h->launches = 0;
     }
+    // (after the pipeline, whose chunks need less room than the whole batch)
+    const bool probe = probe_room(h, n, t);
+    if (!probe && h->stage.cap < (1u << 20)) RK(h->stage.ensure(1u << 20));
     // device-side destination of the CSR offsets
     uint64_t* d_off;
     if (!d.arena && on_device) {

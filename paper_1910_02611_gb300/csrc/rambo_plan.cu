@@ -12,6 +12,7 @@
 // streams against the same (read-only) index.
 #include <cstring>
 #include <new>
+#include <utility>
 
 #include "k_query.cuh"
 #include "rambo_impl.cuh"
@@ -259,26 +260,6 @@ int rambo_plan_create(rambo_t* h, int kind, uint64_t max_queries, uint64_t max_i
         set_staging(form, ix.K, t.staging);
         if (form.bits_words && max_queries <= max_ids / form.bits_min) p->stage_words = max_queries * form.bits_min;
     }
-    // On the probe path every answer is staged as a bitmap of set_pitch(K)
-    // words.  It is taken when an arena for max_queries of them is no more
-    // than four times the one above, or 256 MiB, and memory holds it.
-    const uint64_t pitch = set_pitch(ix.K), plain_words = p->stage_words;
-    const uint64_t most = plain_words * 4 > (64ull << 20) ? plain_words * 4 : 64ull << 20;
-    if (t.set.qw && max_queries <= most / pitch) {
-        const uint64_t words = max_queries * pitch;
-        p->probe = cudaSetDevice(p->device) == cudaSuccess && cudaMalloc(&p->stage, words * 4) == cudaSuccess &&
-                   cudaMalloc(&p->dmask, max_queries * ix.R * ix.S * 4) == cudaSuccess &&
-                   cudaMalloc(&p->dq, max_queries * 8) == cudaSuccess;
-        if (p->probe) {
-            p->stage_words = words;
-        } else {
-            cudaGetLastError();
-            for (uint32_t** d : {&p->stage, &p->dmask, &p->dq}) {
-                if (*d) cudaFree(*d);
-                *d = nullptr;
-            }
-        }
-    }
     p->elem = kind == 0 ? 8 : 1;
     auto fail = [&](int code) {
         plan_free(p);
@@ -292,7 +273,7 @@ int rambo_plan_create(rambo_t* h, int kind, uint64_t max_queries, uint64_t max_i
               cudaMalloc(&p->qcount, max_queries * 4) == cudaSuccess &&
               cudaMalloc(&p->qstart, max_queries * 8) == cudaSuccess &&
               cudaMalloc(&p->scan_tmp, scan_tmp_words(max_queries) * 8) == cudaSuccess &&
-              (p->stage || cudaMalloc(&p->stage, p->stage_words * 4) == cudaSuccess) && cudaMalloc(&p->ids, max_ids * 4) == cudaSuccess &&
+              cudaMalloc(&p->stage, p->stage_words * 4) == cudaSuccess && cudaMalloc(&p->ids, max_ids * 4) == cudaSuccess &&
               cudaMalloc(&p->id_off, (max_queries + 1) * 8) == cudaSuccess &&
               cudaMalloc(&p->d_head, sizeof(PlanHead)) == cudaSuccess &&
               cudaMallocHost(&p->h_data, max_items * p->elem + 16) == cudaSuccess &&
@@ -304,6 +285,31 @@ int rambo_plan_create(rambo_t* h, int kind, uint64_t max_queries, uint64_t max_i
     if (!ok) {
         cudaGetLastError();
         return fail(RAMBO_ENOMEM);
+    }
+    // On the probe path every answer is staged as a bitmap of set_pitch(K)
+    // words and handed over as R * S words of masks.  It is taken when an
+    // arena and masks for max_queries of them are no more than four times the
+    // arena above (or 256 MiB) and a quarter of the memory that is free now
+    // that the plan has all it needs without them; they then take the arena's
+    // place.
+    const uint64_t words = max_queries * set_pitch(ix.K), masks = max_queries * ix.R * ix.S, extra = words + masks + 2 * max_queries;
+    const uint64_t most = p->stage_words * 4 > (64ull << 20) ? p->stage_words * 4 : 64ull << 20;
+    size_t free_b = 0, total_b = 0;
+    if (t.set.qw && extra <= most && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && extra <= (uint64_t)free_b / 16) {
+        uint32_t* stage = nullptr;
+        p->probe = cudaMalloc(&stage, words * 4) == cudaSuccess && cudaMalloc(&p->dmask, masks * 4) == cudaSuccess &&
+                   cudaMalloc(&p->dq, max_queries * 8) == cudaSuccess;
+        if (p->probe) {
+            std::swap(stage, p->stage);
+            p->stage_words = words;
+        } else {
+            cudaGetLastError();
+            for (uint32_t** d : {&p->dmask, &p->dq}) {
+                if (*d) cudaFree(*d);
+                *d = nullptr;
+            }
+        }
+        if (stage) cudaFree(stage);
     }
     p->st = &p->d_head->st;
     p->d_desc = p->d_head->desc;

@@ -1,0 +1,73 @@
+"""Device memory that queries and plans keep, on a runtime without a GPU: the
+bitmaps and masks of a batch are bounded by a quarter of the free memory, the
+masks of wide layouts (hundreds of times their bitmaps) among them, and a plan
+that can be made without them is made."""
+import numpy as np
+import pytest
+
+from tests.fakecuda import Fake
+
+MIB = 1 << 20
+ENOMEM = -4
+
+
+@pytest.fixture(scope="module")
+def fake():
+    return Fake()
+
+
+def _keys(n):
+    return np.arange(n, dtype=np.uint64), np.arange(n + 1, dtype=np.uint64)
+
+
+# 384 bytes of bitmap and 100 KB of masks a query; 250 KB of bitmap and 2 KB of masks
+@pytest.mark.parametrize("K,B,R", [(3000, 50_000, 16), (2_000_000, 500, 8)])
+@pytest.mark.parametrize("on_device", [False, True])
+def test_a_batch_keeps_a_quarter_of_the_free_memory_at_most(fake, K, B, R, on_device):
+    fake.budget(0, 64 << 30)
+    h = fake.create(K, B, R, 64)
+    base = fake.used()
+    fake.budget(0, base + 8192 * MIB)
+    for n in (100, 30_000, 70_000, 70_000):  # (the last two are cut into chunks when they come from the host)
+        assert fake.query(h, *_keys(n), on_device) == 0
+        assert fake.used() - base < 2048 * MIB + 64 * MIB, (n, fake.used() - base)
+    fake.lib.rambo_destroy(h)
+
+
+@pytest.mark.parametrize("K,B,R", [(3000, 50_000, 16), (2_000_000, 500, 8), (1000, 64, 4)])
+def test_a_plan_keeps_a_quarter_of_the_free_memory_at_most_beside_what_it_needs(fake, K, B, R):
+    """A plan of the query kernel alone shows what one needs in any case."""
+    fake.budget(0, 64 << 30)
+    h = fake.create(K, B, R, 64)
+    cfg = _config(fake, h)
+    for n, ids in ((1000, 1 << 20), (20_000, 1 << 27), (200_000, 1 << 27)):
+        fake.budget(0, 64 << 30)
+        cfg.set_stage, cfg.row_load = int(B > 4096), 0
+        assert fake.lib.rambo_set_query_config(h, cfg) == 0
+        base = fake.used()
+        rc, p = fake.plan(h, 0, n, 4 * n, ids)
+        assert rc == 0
+        need = fake.used() - base
+        fake.lib.rambo_plan_destroy(p)
+        assert fake.used() == base
+        cfg.set_stage, cfg.row_load = 0, 7
+        assert fake.lib.rambo_set_query_config(h, cfg) == 0
+        for room in (need, need + 100 * MIB, 3 * need, 64 << 30):
+            fake.budget(0, base + room)
+            rc, p = fake.plan(h, 0, n, 4 * n, ids)
+            assert rc == 0, (n, ids, room, need)
+            assert fake.used() - base <= need + room // 4, (n, ids, room, need, fake.used() - base)
+            fake.lib.rambo_plan_destroy(p)
+            assert fake.used() == base
+        fake.budget(0, base + need - MIB)
+        assert fake.plan(h, 0, n, 4 * n, ids)[0] == ENOMEM
+        assert fake.used() == base
+    fake.lib.rambo_destroy(h)
+
+
+def _config(fake, h):
+    from paper_1910_02611_gb300.rambo import QueryConfig
+
+    cfg = QueryConfig()
+    assert fake.lib.rambo_get_query_config(h, cfg) == 0
+    return cfg
