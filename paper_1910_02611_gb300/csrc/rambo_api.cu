@@ -1107,10 +1107,12 @@ int settle_times(rambo* h) {
 namespace rgb {
 // Read-only view of a handle for the fixed-scratch query entry point
 // (rambo_noalloc.cu): index, hash parameters and the kernel tuning the handle
-// would use for n queries.  Allocates nothing.
+// would use for n queries.  Allocates nothing; the handle's device is current
+// afterwards.
 int handle_query_view(rambo_t* h, uint64_t n, IndexView* ix, HashParams* hp, QueryTuning* t, int* use_bitmap,
                       int* device) {
     if (!h || !ix || !hp || !t || !use_bitmap || !device) return RAMBO_EINVAL;
+    CK(cudaSetDevice(h->device));  // (what the tuning asks of the kernels holds for the current device)
     RK(resolve_tuning(h, n, *use_bitmap, *t));
     *ix = h->view();
     *hp = h->hp;
