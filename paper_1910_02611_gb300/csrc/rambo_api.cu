@@ -159,14 +159,16 @@ struct rambo {
     uint64_t launches = 0;
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};  // call start, query start/end, call end
     uint64_t last_err_item = 0;
-    // block sizes and residency resolved for the query configuration tuned_cfg
+    // block sizes and residency resolved for the query configuration
+    // tuned_cfg: the query kernel's, and once a call asks for them the probe
+    // and set kernels'
     struct Tuned {
         int wpb = 0, per_sm = 0, per_sm_g = 0;                    // query kernel
         int probe_wpb = 0, probe_per_sm = 0, probe_per_sm_g = 0, probe_per_sm_l = 0;  // probe kernel
         SetLaunch set{};
     } tuned;
     rambo_query_config_t tuned_cfg{};
-    bool tuned_known = false;
+    bool tuned_known = false, probe_known = false;
     std::vector<rambo_plan_t*> plans;   // live plans (own or a server's) holding captured pointers
     unsigned char* na_base = nullptr;   // device address of the no-alloc query's fixed scratch
 
@@ -558,9 +560,9 @@ bool pick_block(F per_sm_of, int& wpb, int& per_sm) {
     return false;
 }
 
-// Block sizes and blocks per SM of the kernels for the handle's configuration,
-// kept until the configuration changes (the occupancy queries behind them
-// cost more than a small batch's kernels).
+// Block sizes and blocks per SM of the query kernel for the handle's
+// configuration, kept until the configuration changes (the occupancy queries
+// behind them cost more than a small batch's kernels).
 int resolve_residency(rambo* h, int use_bitmap) {
     const int V = (int)h->cfg.words_per_lane, G = (int)h->cfg.lanes_per_key;
     rambo::Tuned u{};
@@ -582,6 +584,18 @@ int resolve_residency(rambo* h, int use_bitmap) {
     if (use_bitmap && group != 1 && u.wpb > 1)
         u.per_sm_g = std::min(most, query_max_blocks_per_sm(V, G, h->eta, true, u.wpb,
                                                             query_group_smem_bytes(h->R, h->S, h->K, u.wpb, group)));
+    h->tuned = u;
+    h->tuned_cfg = h->cfg;
+    h->tuned_known = true;
+    h->probe_known = false;
+    return RAMBO_OK;
+}
+
+// The probe and set kernels' counterparts, kept with them.
+void resolve_probe(rambo* h) {
+    const int V = (int)h->cfg.words_per_lane, G = (int)h->cfg.lanes_per_key, group = (int)h->cfg.warps_per_query;
+    rambo::Tuned& u = h->tuned;
+    const int most = h->cfg.blocks_per_sm ? (int)h->cfg.blocks_per_sm : 1 << 20;
     // the probe and set kernels serve the automatic set stage and staging form
     // and the default row reads; other choices name what the query kernel does
     if (h->cfg.set_stage == 0 && h->cfg.answer_staging == 0 && h->cfg.row_load == 7) u.set = set_launch_shape(h->view(), h->num_sms);
@@ -603,10 +617,7 @@ int resolve_residency(rambo* h, int use_bitmap) {
             u.probe_per_sm_g = std::min(most, probe_max_blocks_per_sm(V, G, h->eta, PB_GROUP, u.probe_wpb,
                                                                       probe_group_smem_bytes(h->R, h->S, u.probe_wpb)));
     }
-    h->tuned = u;
-    h->tuned_cfg = h->cfg;
-    h->tuned_known = true;
-    return RAMBO_OK;
+    h->probe_known = true;
 }
 
 // Queries a warp takes per work-queue ticket.
@@ -615,7 +626,10 @@ int ticket_batch(uint64_t n, uint64_t warps) {
     return (int)(batch < 1 ? 1 : batch > 16 ? 16 : batch);
 }
 
-int resolve_tuning(rambo* h, uint64_t n, int& use_bitmap, QueryTuning& t) {
+// The kernels' launches for a batch of n queries.  probe = false: of the query
+// kernel alone, without a question about the probe and set kernels (the first
+// one would load them).
+int resolve_tuning(rambo* h, uint64_t n, int& use_bitmap, QueryTuning& t, bool probe = true) {
     t = QueryTuning{};
     if (query_is_wide(h->R, h->S)) {
         // rows wider than the register tiling or more than RF tables: one
@@ -626,14 +640,18 @@ int resolve_tuning(rambo* h, uint64_t n, int& use_bitmap, QueryTuning& t) {
         if (!h->tuned_known) {
             h->tuned = rambo::Tuned{};
             h->tuned.per_sm = query_wide_blocks_per_sm(h->R, h->S, h->eta);
-            h->tuned.set = set_launch_shape(h->view(), h->num_sms);
             h->tuned_known = true;
+            h->probe_known = false;
+        }
+        if (probe && !h->probe_known) {
+            h->tuned.set = set_launch_shape(h->view(), h->num_sms);
+            h->probe_known = true;
         }
         if (h->tuned.per_sm < 1) return RAMBO_EINVAL;
         uint64_t blocks = (uint64_t)h->tuned.per_sm * h->num_sms;
         if (blocks > n) blocks = n;
         t.blocks = (int)(blocks < 1 ? 1 : blocks);
-        if (h->cfg.set_stage == 0 && h->cfg.answer_staging == 0) t.set = h->tuned.set;
+        if (probe && h->cfg.set_stage == 0 && h->cfg.answer_staging == 0) t.set = h->tuned.set;
         t.warps_per_block = QW_THREADS / 32;
         t.batch = 1;
         return RAMBO_OK;
@@ -647,6 +665,7 @@ int resolve_tuning(rambo* h, uint64_t n, int& use_bitmap, QueryTuning& t) {
     t.group = (int)h->cfg.warps_per_query;
     use_bitmap = (h->mem_off && t.set_stage != 1 && (h->K + 31) / 32 <= 4096) ? 1 : 0;
     if (!h->tuned_known || std::memcmp(&h->tuned_cfg, &h->cfg, sizeof(h->cfg)) != 0) RK(resolve_residency(h, use_bitmap));
+    if (probe && !h->probe_known) resolve_probe(h);
     const rambo::Tuned& u = h->tuned;
     t.warps_per_block = u.wpb;
     uint64_t blocks = (uint64_t)u.per_sm * h->num_sms;
@@ -660,7 +679,7 @@ int resolve_tuning(rambo* h, uint64_t n, int& use_bitmap, QueryTuning& t) {
     t.blocks_group = (int)bg;
     t.group_warps = bg * (uint64_t)t.warps_per_block;
     t.batch = ticket_batch(n, blocks * t.warps_per_block);
-    if (u.set.qw) {
+    if (probe && u.set.qw) {
         t.set = u.set;
         t.probe_warps = u.probe_wpb;
         blocks = (uint64_t)u.probe_per_sm * h->num_sms;
@@ -1105,15 +1124,15 @@ int settle_times(rambo* h) {
 }  // namespace
 
 namespace rgb {
-// Read-only view of a handle for the fixed-scratch query entry point
+// Read-only view of a handle for plans and the fixed-scratch query entry point
 // (rambo_noalloc.cu): index, hash parameters and the kernel tuning the handle
-// would use for n queries.  Allocates nothing; the handle's device is current
-// afterwards.
+// would use for n queries (probe = false: on the query kernel).  Allocates
+// nothing; the handle's device is current afterwards.
 int handle_query_view(rambo_t* h, uint64_t n, IndexView* ix, HashParams* hp, QueryTuning* t, int* use_bitmap,
-                      int* device) {
+                      int* device, bool probe) {
     if (!h || !ix || !hp || !t || !use_bitmap || !device) return RAMBO_EINVAL;
     CK(cudaSetDevice(h->device));  // (what the tuning asks of the kernels holds for the current device)
-    RK(resolve_tuning(h, n, *use_bitmap, *t));
+    RK(resolve_tuning(h, n, *use_bitmap, *t, probe));
     *ix = h->view();
     *hp = h->hp;
     *device = h->device;

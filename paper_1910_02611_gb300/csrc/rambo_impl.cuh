@@ -469,9 +469,10 @@ cudaError_t launch_query_one(const IndexView& ix, const HashParams& hp, int seq,
                              const uint64_t* keys, uint64_t len, uint32_t k, int canon, int skipn, uint32_t* out_ids,
                              uint32_t* out_count, int* bad, cudaStream_t s);
 
-// rambo_api.cu: what the fixed-scratch entry point needs from a handle
+// rambo_api.cu: what plans and the fixed-scratch entry point (which runs the
+// query kernel alone: probe = false) need from a handle
 int handle_query_view(rambo_t* h, uint64_t n, IndexView* ix, HashParams* hp, QueryTuning* t, int* use_bitmap,
-                      int* device);
+                      int* device, bool probe);
 // rambo_api.cu: plans hold device pointers of their handle inside a captured
 // graph; the handle keeps a list of them, refuses calls that would move those
 // buffers while any is alive, and orphans them (plan_orphan, rambo_plan.cu)

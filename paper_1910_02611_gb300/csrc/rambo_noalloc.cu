@@ -116,7 +116,7 @@ extern "C" int rambo_query_seq_batch_noalloc(rambo_t* h, const uint8_t* bases, c
     HashParams hp;
     QueryTuning t;
     int use_bitmap = 0, dev = 0;
-    int rc = handle_query_view(h, n ? n : 1, &ix, &hp, &t, &use_bitmap, &dev);
+    int rc = handle_query_view(h, n ? n : 1, &ix, &hp, &t, &use_bitmap, &dev, false);
     if (rc) return rc;
     NA_CK(cudaSetDevice(dev));
     unsigned char* base = handle_noalloc_base(h);

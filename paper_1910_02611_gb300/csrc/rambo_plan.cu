@@ -131,7 +131,7 @@ int plan_capture(rambo_plan* p, bool timed) {
     HashParams hp;
     QueryTuning t;
     int use_bitmap = 0, dev = 0;
-    int rc = handle_query_view(p->h, p->max_q, &ix, &hp, &t, &use_bitmap, &dev);
+    int rc = handle_query_view(p->h, p->max_q, &ix, &hp, &t, &use_bitmap, &dev, true);
     if (rc) return rc;
     BatchView b{};
     b.seq = p->kind;
@@ -238,7 +238,7 @@ int rambo_plan_create(rambo_t* h, int kind, uint64_t max_queries, uint64_t max_i
     HashParams hp;
     QueryTuning t;
     int ub = 0;
-    int rc = handle_query_view(h, max_queries, &ix, &hp, &t, &ub, &p->device);
+    int rc = handle_query_view(h, max_queries, &ix, &hp, &t, &ub, &p->device, true);
     if (rc) {
         delete p;
         return rc;

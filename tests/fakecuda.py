@@ -69,6 +69,13 @@ class Fake:
         assert self.lib.rambo_create(K, B, R, m, eta, seed, C.byref(h)) == 0
         return h
 
+    def config(self, h):
+        from paper_1910_02611_gb300.rambo import QueryConfig
+
+        cfg = QueryConfig()
+        assert self.lib.rambo_get_query_config(h, cfg) == 0
+        return cfg
+
     def query(self, h, data: np.ndarray, offsets: np.ndarray, on_device: bool, k: int = 31) -> int:
         """The arena call, for keys or (bytes) sequences; `device` memory is host memory here."""
         ids, off = C.c_void_p(), C.c_void_p()

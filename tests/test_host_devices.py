@@ -1,6 +1,7 @@
 """What the host code asks of the kernels, and where, on a runtime without a
 GPU (two devices): a handle's kernels are set up on the handle's device
-whichever is current."""
+whichever is current, and the query that promises to load no code asks nothing
+of kernels that creating the handle did not load."""
 import numpy as np
 import pytest
 
@@ -35,4 +36,36 @@ def test_a_handle_is_set_up_on_its_own_device(fake, K, B, R, first):
     assert all(e["device"] == 0 for e in events), [e for e in events if e["device"]]
     if plan:
         fake.lib.rambo_plan_destroy(plan)
+    fake.lib.rambo_destroy(h)
+
+
+@pytest.mark.parametrize("K,B,R,eta", [(5000, 1000, 8, 2), (5000, 20_000, 4, 1), (300, 40, 3, 3), (200_000, 64, 5, 4)])
+def test_a_no_alloc_query_uses_only_kernels_that_creation_loaded(fake, K, B, R, eta):
+    """Under lazy loading the first use of a kernel loads it, be it a question about its occupancy."""
+    fake.device(0)
+    fake.clear()
+    h = fake.create(K, B, R, 64, eta)
+    loaded = {e["name"] for e in fake.events("LF")}
+    bases, ends = np.full(6200, ord("A"), np.uint8), np.arange(0, 6201, 31, dtype=np.uint64)
+    for change in (None, "config", "fold", None):
+        if change == "config":
+            cfg = fake.config(h)
+            cfg.visit_order = 1
+            cfg.blocks_per_sm = 1
+            assert fake.lib.rambo_set_query_config(h, cfg) == 0
+        elif change == "fold":
+            fake.clear()
+            assert fake.lib.rambo_fold(h, None) == 0
+            loaded |= {e["name"] for e in fake.events("LF")}
+        for n in (200, 1):
+            fake.clear()
+            assert fake.noalloc(h, bases, ends[: n + 1]) == 0
+            events = fake.events()
+            assert any(e["kind"] == "L" for e in events)
+            assert {e["name"] for e in events if e["name"]} <= loaded
+            assert not any(e["kind"] == "M" for e in events)
+        # what the no-alloc call resolved is not all that an ordinary query needs
+        if change is None:
+            assert fake.query(h, np.arange(2000, dtype=np.uint64), np.arange(2001, dtype=np.uint64), False) == 0
+            assert any("k_set" in e["name"] for e in fake.events("L"))
     fake.lib.rambo_destroy(h)
