@@ -266,12 +266,12 @@ cudaError_t launch_intake(const BatchView& b, uint64_t min_len, uint64_t K, cons
                           uint64_t n_words, uint32_t* nmask, DevStatus* st, cudaStream_t s) {
     if (b.n == 0 && !b.desc) return cudaSuccess;
     const unsigned prio = b.seq ? PRIO_EBADSEQ : PRIO_EINVAL;
-    const uint64_t work = b.n > n_words ? b.n : n_words;  // capacities for a descriptor batch
-    // a batch sized on the device: for eight words a query, 64 blocks at least
-    // (one long sequence) and one resident wave at most
-    const int blocks = !b.ends ? grid_for(work, 256, 1 << 16)
-                       : bases ? std::max(64, grid_for(b.n * 8, 256, 152 * 8))
-                               : grid_for(b.n, 256, 152 * 8);
+    const uint64_t work = b.n > n_words ? b.n : n_words;  // capacities for a batch sized on the device
+    // a batch sized on the device fills the room it has been given at most, and
+    // one resident wave serves it: how long its sequences are is not known here.
+    // 5e8 bases in 1 or 100 of them, a call: 215-225 us; with a grid by the
+    // number of queries (64 blocks) 930.  300 bases: 56 us with either.
+    const int blocks = grid_for(work, 256, b.ends ? 152 * 8 : 1 << 16);
     k_intake<<<blocks, 256, 0, s>>>(b, min_len, prio, K, bases, packed, n_words, nmask, st);
     return cudaGetLastError();
 }

@@ -69,3 +69,16 @@ def test_a_no_alloc_query_uses_only_kernels_that_creation_loaded(fake, K, B, R, 
             assert fake.query(h, np.arange(2000, dtype=np.uint64), np.arange(2001, dtype=np.uint64), False) == 0
             assert any("k_set" in e["name"] for e in fake.events("L"))
     fake.lib.rambo_destroy(h)
+
+
+@pytest.mark.parametrize("n,bases", [(1, 3_000_000), (7, 3_000_000), (1, 20_000_000), (300, 3_000_000)])
+def test_long_sequences_on_the_device_are_packed_by_enough_blocks(fake, n, bases):
+    fake.device(0)
+    h = fake.create(300, 40, 3, 64)
+    data, ends = np.full(bases, ord("A"), np.uint8), np.linspace(0, bases, n + 1).astype(np.uint64)
+    for _ in range(2):  # (a handle's first sequences are sized on the host, later ones on the device)
+        fake.clear()
+        assert fake.query(h, data, ends, True) == 0
+        (intake,) = [e for e in fake.events("L") if "k_intake" in e["name"]]
+        assert intake["grid"] >= min(8 * 152, bases // 32 // 256), intake
+    fake.lib.rambo_destroy(h)
