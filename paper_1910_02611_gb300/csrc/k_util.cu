@@ -589,6 +589,14 @@ cudaError_t launch_cluster_order(const BatchView& b, uint64_t* keys, uint32_t* h
 // (2e9 IDs, 8 GB) 1.76 -> 1.65 ms.  Parts of 2048 words: 4096 measured 5%
 // slower on the last of these, 512 and 1024 slower on the one before it.
 //
+// Since every part counts from the start of its bitmap, the number of parts
+// is bounded (GA_PARTS_*), or the counting grows with the square of K: at K =
+// 1e7 the gather of 500 answers of 1e7 IDs took 6.1 ms with parts of a fixed
+// length and 3.8 with eight, of 256 answers of one ID 4.3 ms (one warp each,
+// since parts of that length filled the grid) and 0.57.  A few answers like
+// the parts short: 1 of 1e7 IDs 279 us unbounded, 315 with 128 parts, 363
+// with 64.
+//
 // A query staged as its K-bit bitmap is expanded 32 words (up to 1024 IDs) at
 // a time: every lane writes its word's set bits as IDs into the warp's run in
 // shared memory at its prefix position, then the warp stores the run 16 bytes
@@ -602,6 +610,8 @@ constexpr int GA_RUN = 1024;                  // IDs of 32 bitmap words
 constexpr uint32_t GA_SHORT = 4096;           // answers of at most this many IDs are not cut where the grid is filled
 constexpr uint32_t GA_PART_WORDS = 2048;     // bitmap words of a part in a batch that fills the grid,
 constexpr uint32_t GA_PART_LEAST = 128;       // and of the smallest part where it does not
+constexpr uint32_t GA_PARTS_FILLED = 8;       // most parts in a batch that fills the grid,
+constexpr uint32_t GA_PARTS_MOST = 128;       // and in one that does not
 constexpr unsigned GA_TAKE = 8;               // most parts per work-queue ticket
 
 // entry p of a run: four pad words per 32, so lanes whose words are all full
@@ -715,12 +725,18 @@ __device__ __forceinline__ uint32_t ga_count(const uint32_t* __restrict__ src, u
     return c;
 }
 
+// Most parts a long answer is cut into.
+__host__ __device__ inline uint32_t ga_parts_most(uint32_t bits_words) {
+    const uint32_t parts = (bits_words + GA_PART_LEAST - 1) / GA_PART_LEAST;
+    return !bits_words ? 16 : parts < GA_PARTS_MOST ? parts : GA_PARTS_MOST;
+}
+
 // Parts a long answer is cut into when n queries share a grid of `warps`.
 // Sets the longest answer that stays whole: with warps to spare, none (a few
 // IDs spread over 1e5 bits kept one warp for 50 us).
 __device__ __forceinline__ uint32_t ga_parts(uint32_t bits_words, uint64_t n, uint64_t warps, uint32_t& whole) {
-    const uint32_t base = bits_words ? (bits_words + GA_PART_WORDS - 1) / GA_PART_WORDS : 4;
-    const uint32_t most = bits_words ? (bits_words + GA_PART_LEAST - 1) / GA_PART_LEAST : 16;
+    const uint32_t base = bits_words ? min((bits_words + GA_PART_WORDS - 1) / GA_PART_WORDS, GA_PARTS_FILLED) : 4;
+    const uint32_t most = ga_parts_most(bits_words);
     const uint64_t fill = warps / n;  // parts that occupy every warp
     const uint32_t parts = fill < most ? (uint32_t)fill : most;
     whole = parts > base ? 0 : GA_SHORT;
@@ -803,7 +819,7 @@ cudaError_t launch_gather(const QueryOut& o, const uint64_t* id_offsets, uint64_
     }
     // (no more warps than the smallest parts of n answers)
     const uint64_t most = dev < 64 ? wave[dev] : 152 * 4;
-    const uint64_t parts = o.bits_words ? (o.bits_words + GA_PART_LEAST - 1) / GA_PART_LEAST : 16;
+    const uint64_t parts = ga_parts_most(o.bits_words);
     const uint64_t want = n >= most * GA_WARPS ? most : (n * parts + GA_WARPS - 1) / GA_WARPS;
     const uint64_t blocks = std::min(most, want);
     k_gather<<<(unsigned)blocks, GA_THREADS, 0, s>>>(o, id_offsets, n, ids, st, n_dev, ids_cap);

@@ -82,3 +82,16 @@ def test_long_sequences_on_the_device_are_packed_by_enough_blocks(fake, n, bases
         (intake,) = [e for e in fake.events("L") if "k_intake" in e["name"]]
         assert intake["grid"] >= min(8 * 152, bases // 32 // 256), intake
     fake.lib.rambo_destroy(h)
+
+
+@pytest.mark.parametrize("K", [10_000_000, 500_000_000])
+def test_the_gather_of_one_answer_is_cut_into_a_bounded_number_of_parts(fake, K):
+    """Every part counts its bitmap from the start, so their number is the number of times it is read."""
+    fake.device(0)
+    h = fake.create(K, 2000, 2, 64)
+    for n in (1, 3):
+        fake.clear()
+        assert fake.query(h, np.arange(n, dtype=np.uint64), np.arange(n + 1, dtype=np.uint64), False) == 0
+        (gather,) = [e for e in fake.events("L") if "k_gather" in e["name"]]
+        assert gather["grid"] * 8 <= 128 * n + 8, gather  # (eight warps a block, a part each)
+    fake.lib.rambo_destroy(h)
