@@ -588,6 +588,10 @@ cudaError_t launch_cluster_order(const BatchView& b, uint64_t* keys, uint32_t* h
 // documents (9.8e8 IDs; staged as lists before) 11.8 -> 0.93 ms, 1e5 over 1e5
 // (2e9 IDs, 8 GB) 1.76 -> 1.65 ms.  Parts of 2048 words: 4096 measured 5%
 // slower on the last of these, 512 and 1024 slower on the one before it.
+// Smallest parts of 64 words, and no more answers a take than leaves every
+// warp some: 64 queries over 4000 sets, 2000 IDs each, 46 us with parts of 128
+// words, 20 with 64 or 32 (2000 of one ID 28, 22, 24); 64 over 1000 sets, 500
+// IDs each, 31 us by eight a take, 19 by one.
 //
 // Since every part counts from the start of its bitmap, the number of parts
 // is bounded (GA_PARTS_*), or the counting grows with the square of K: at K =
@@ -609,7 +613,7 @@ constexpr int GA_WARPS = GA_THREADS / 32;
 constexpr int GA_RUN = 1024;                  // IDs of 32 bitmap words
 constexpr uint32_t GA_SHORT = 4096;           // answers of at most this many IDs are not cut where the grid is filled
 constexpr uint32_t GA_PART_WORDS = 2048;     // bitmap words of a part in a batch that fills the grid,
-constexpr uint32_t GA_PART_LEAST = 128;       // and of the smallest part where it does not
+constexpr uint32_t GA_PART_LEAST = 64;        // and of the smallest part where it does not
 constexpr uint32_t GA_PARTS_FILLED = 8;       // most parts in a batch that fills the grid,
 constexpr uint32_t GA_PARTS_MOST = 128;       // and in one that does not
 constexpr unsigned GA_TAKE = 8;               // most parts per work-queue ticket
@@ -757,8 +761,11 @@ __global__ void __launch_bounds__(GA_THREADS, 6) k_gather(QueryOut o, const uint
     const uint32_t parts = ga_parts(o.bits_words, n, warps, whole);
     const uint64_t units = n * parts;
     // answers that are cut into many parts are taken a part at a time, so that
-    // a long one's parts go to several warps; the first take needs no ticket
-    const unsigned take = parts == 1 ? GA_TAKE : parts < 8 && units >= warps * GA_TAKE ? GA_TAKE / 2 : 1;
+    // a long one's parts go to several warps, and whole ones no more at a time
+    // than leaves every warp some; the first take needs no ticket
+    const unsigned take = units >= warps * GA_TAKE ? (parts == 1 ? GA_TAKE : parts < 8 ? GA_TAKE / 2 : 1)
+                          : parts == 1             ? max(1u, (unsigned)(units / warps))
+                                                   : 1;
     for (unsigned long long u0 = ((uint64_t)blockIdx.x * GA_WARPS + (threadIdx.x >> 5)) * take; u0 < units;) {
         // a lane looks up each unit of the ticket, then the warp takes them one by one
         uint32_t c_of = 0, part_of = 0;
