@@ -765,8 +765,10 @@ int enqueue_intake(rambo* h, BatchView& b, const void* d_data, int seq, uint32_t
     uint64_t n_words = 0;
     b.nmask = nullptr;
     if (seq) {
-        // (sized on the device: as many words as there are; the intake says so when they are too few)
-        n_words = b.ends ? h->packed.cap : b.total / 32 + 2;  // one spare word for windows crossing the last word
+        n_words = b.total / 32 + 2;  // one spare word for windows crossing the last word
+        // sized on the device: as many words as there are, of the packed bases
+        // and the mask; the intake says so when they are too few
+        if (b.ends) n_words = b.skipn ? std::min(h->packed.cap, h->nmask.cap) : h->packed.cap;
         RK(h->packed.ensure(n_words));
         b.packed = h->packed.p;
         if (b.skipn) {
@@ -958,7 +960,7 @@ int run_query(rambo* h, int seq, const void* data, const uint64_t* offsets, uint
     RK(h->qcount.ensure(n));
     RK(h->qstart.ensure(n));
     RK(h->scan_tmp.ensure(scan_tmp_words(n)));
-    if (on_device && !h->cfg.cluster && (!seq || h->packed.p)) {
+    if (on_device && !h->cfg.cluster && (!seq || h->packed.p) && (!skipn || h->nmask.p)) {
         // the kernels read where the batch starts and ends; nothing waits for it here
         b.n = n;
         b.offsets = offsets;
@@ -1045,8 +1047,9 @@ int run_query(rambo* h, int seq, const void* data, const uint64_t* offsets, uint
         }
         CK(cudaStreamSynchronize(s));
         if (h->h_st->err != NO_ERR && (h->h_st->err & 0xff) == PRIO_GROW) {
-            // a batch sized on the device that the packed buffer does not hold: grow it and run again
+            // a batch sized on the device that the packed buffer (or the mask) does not hold: grow it and run again
             RK(h->packed.ensure(h->h_st->total / 32 + 2));
+            if (skipn) RK(h->nmask.ensure(h->h_st->total / 32 + 2));
             h->launches = 0;
             continue;
         }

@@ -80,3 +80,15 @@ def test_offsets_outside_the_batch_are_refused(work):
     ids, off = _device(g, one.data, one.offsets, k)
     assert np.array_equal(off, want[1]) and np.array_equal(ids, want[0])
     g.close()
+
+
+def test_the_mask_grows_by_itself(work):
+    """After a large batch without a mask, a small and a large one with it."""
+    fresh, o, plain, q = work
+    g = fresh()
+    for k, n in ((31, 1000), (31 | SKIP_N, 1), (31, 1000), (31 | SKIP_N, 1000), (31 | SKIP_N, 999), (31, 1000)):
+        part = (q if k & SKIP_N else plain).subset(np.arange(n))
+        want = o.query_batch("seq", part.data, part.offsets, k=k)
+        ids, off = _device(g, part.data, part.offsets, k)
+        assert np.array_equal(off, want[1]) and np.array_equal(ids, want[0])
+    g.close()

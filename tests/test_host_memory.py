@@ -65,6 +65,19 @@ def test_a_plan_keeps_a_quarter_of_the_free_memory_at_most_beside_what_it_needs(
     fake.lib.rambo_destroy(h)
 
 
+def test_a_skip_n_batch_does_not_allocate_a_mask_for_the_largest_batch_before_it(fake):
+    fake.budget(0, 64 << 30)
+    h = fake.create(1000, 64, 4, 64)
+    data, ends = np.full(200_000_000, ord("A"), np.uint8), lambda n: np.array([0, n], np.uint64)
+    for _ in range(2):
+        assert fake.query(h, data, ends(data.size), True) == 0
+    base = fake.used()
+    for n in (400, 4000, 40_000):
+        assert fake.query(h, data, ends(n), True, 31 | 0x200) == 0
+    assert fake.used() - base < MIB
+    fake.lib.rambo_destroy(h)
+
+
 def _config(fake, h):
     from paper_1910_02611_gb300.rambo import QueryConfig
 
