@@ -107,3 +107,15 @@ def test_answers_over_a_few_thousand_sets_take_several_warps(fake, K, parts):
     (gather,) = [e for e in fake.events("L") if "k_gather" in e["name"]]
     assert gather["grid"] == 64 * parts // 8, gather
     fake.lib.rambo_destroy(h)
+
+
+@pytest.mark.parametrize("n,terms,modes", [(2047, 1, "0"), (2048, 1, "2"), (2048, 8, "02"), (2048, 9, "0"), (300, 400, "1")])
+def test_the_probe_instance_of_a_host_batch(fake, n, terms, modes):
+    """0 a warp a query, 1 several warps, 2 lane groups (and a warp for the long ones, if there can be one)."""
+    fake.device(0)
+    h = fake.create(5000, 500, 4, 64)
+    fake.clear()
+    assert fake.query(h, np.arange(n * terms, dtype=np.uint64), np.arange(0, n * terms + 1, terms, dtype=np.uint64), False) == 0
+    got = {e["name"].split("k_probeI")[1].split("EEEv")[0][-1] for e in fake.events("L") if "k_probeI" in e["name"]}
+    assert got == set(modes), got
+    fake.lib.rambo_destroy(h)
