@@ -109,7 +109,7 @@ def test_answers_over_a_few_thousand_sets_take_several_warps(fake, K, parts):
     fake.lib.rambo_destroy(h)
 
 
-@pytest.mark.parametrize("n,terms,modes", [(2047, 1, "0"), (2048, 1, "2"), (2048, 8, "02"), (2048, 9, "0"), (300, 400, "1")])
+@pytest.mark.parametrize("n,terms,modes", [(2047, 1, "0"), (2048, 1, "2"), (2048, 8, "02"), (20_000, 9, "0"), (2048, 9, "1"), (300, 400, "1")])
 def test_the_probe_instance_of_a_host_batch(fake, n, terms, modes):
     """0 a warp a query, 1 several warps, 2 lane groups (and a warp for the long ones, if there can be one)."""
     fake.device(0)
