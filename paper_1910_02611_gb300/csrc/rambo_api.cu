@@ -421,7 +421,10 @@ int insert_bucketed(rambo* h, const BatchView& b, cudaStream_t s) {
     // (48 MiB windows measured faster than 32 MiB ones of a power of two of
     // rows: genome 360 vs 485 ms, uneven 730 vs 866 ms)
     uint64_t rows_per_win = BUCKET_WIN_BYTES / ((uint64_t)h->S * 4);
-    if (rows_per_win >= 8192) rows_per_win &= ~4095ull;  // (the scatter's window quotient is then one multiplication)
+    // (whole 4096 rows, as long as there are not too many windows then: the
+    // scatter's window quotient is one multiplication)
+    const uint64_t even = rows_per_win & ~4095ull;
+    if (rows_per_win >= 8192 && (rows_total + even - 1) / even <= 4096) rows_per_win = even;
     if (rows_per_win < 1) rows_per_win = 1;
     if (rows_per_win > rows_total) rows_per_win = rows_total;
     const uint64_t n_win64 = (rows_total + rows_per_win - 1) / rows_per_win;

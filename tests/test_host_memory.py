@@ -78,6 +78,22 @@ def test_a_skip_n_batch_does_not_allocate_a_mask_for_the_largest_batch_before_it
     fake.lib.rambo_destroy(h)
 
 
+@pytest.mark.parametrize("R,m", [(1, 1 << 15), (5, 1 << 23)])  # 135 MB; 172 GB, more than 4096 windows of 8192 rows
+def test_large_builds_are_bucketed_up_to_4096_windows_of_48_mib(fake, R, m):
+    fake.budget(0, 280 << 30)
+    h = fake.create(1000, 32_880, R, m, 2)  # rows of 4112 bytes: 12240 of them in a window
+    n = -(-(1 << 26) // (2 * R)) + 1
+    ids, keys, ends = np.zeros(1, np.uint64), np.zeros(n, np.uint64), np.array([0, n], np.uint64)
+    fake.clear()
+    fake.status(0, 2**64 - 1)
+    assert fake.lib.rambo_insert_batch(h, ids.ctypes.data, keys.ctypes.data, ends.ctypes.data, 1, 0, None) == 0
+    fake.status()
+    names = [e["name"] for e in fake.events("L")]
+    assert any("k_bucket_scatter" in x for x in names) and not any("k_insert" in x for x in names)
+    assert sum("k_bucket_apply" in x for x in names) <= 4096
+    fake.lib.rambo_destroy(h)
+
+
 def _config(fake, h):
     from paper_1910_02611_gb300.rambo import QueryConfig
 
