@@ -3,7 +3,7 @@
 
 namespace rgb {
 
-using ProbeKernel = void (*)(IndexView, HashParams, BatchView, QueryOut, int, int, int, unsigned long long, int,
+using ProbeKernel = void (*)(IndexView, HashParams, BatchView, QueryOut, int, int, int, int, unsigned long long, int,
                              DevStatus*);
 ProbeKernel probe_kernel_e2(int V, int G, int mode);
 ProbeKernel probe_kernel_e4(int V, int G, int mode);
@@ -42,23 +42,23 @@ cudaError_t launch_probe(const IndexView& ix, const HashParams& hp, const BatchV
     // are not worth the third one: they rarely have just eight k-mers).
     const int group = t.probe_blocks_group > 0 ? t.group : 1;
     bool run[3] = {true, t.probe_blocks_group > 0, !(b.desc && b.seq) && group <= 1 && b.n >= PB_MANY};
-    if (b.ends && qk_group_size(b.n, group, (unsigned)t.probe_warps, t.probe_group_warps, 1) == 1) run[PB_GROUP] = false;
+    if (b.ends && qk_group_size(b.n, group, (unsigned)t.probe_group_wpb, t.probe_group_warps, 1) == 1) run[PB_GROUP] = false;
     if (!b.desc && !b.ends) {
         unsigned P;
-        const int mode = probe_mode(b, group, (unsigned)t.probe_warps, t.probe_group_warps, 1, P);
+        const int mode = probe_mode(b, group, (unsigned)t.probe_group_wpb, t.probe_group_warps, 1, P);
         for (int m = 0; m < 3; ++m) run[m] = m == mode;
         // with lane groups, also for queries longer than they take, if there can be one
         const uint64_t least = b.seq ? b.k : 1;
         if (mode == PB_LANES) run[PB_WARP] = b.total > (b.n - 1) * least + (least - 1) + PB_SHORT_MOST;
     }
-    const unsigned threads = (unsigned)t.probe_warps * 32;
     for (const int mode : {PB_LANES, PB_WARP, PB_GROUP}) {
         if (!run[mode]) continue;
         const ProbeKernel f = probe_kernel(t.V, t.G, ix.eta, mode);
         if (!f) return cudaErrorInvalidValue;
-        const size_t smem = mode == PB_GROUP ? probe_group_smem_bytes(ix.R, ix.S, t.probe_warps) : 0;
+        const unsigned threads = (unsigned)(mode == PB_GROUP ? t.probe_group_wpb : t.probe_warps) * 32;
+        const size_t smem = mode == PB_GROUP ? probe_group_smem_bytes(ix.R, ix.S, t.probe_group_wpb) : 0;
         const int blocks = mode == PB_GROUP ? t.probe_blocks_group : mode == PB_LANES ? t.probe_blocks_lanes : t.probe_blocks;
-        f<<<(unsigned)blocks, threads, smem, s>>>(ix, hp, b, o, t.probe_batch, t.order, group,
+        f<<<(unsigned)blocks, threads, smem, s>>>(ix, hp, b, o, t.probe_batch, t.order, group, t.probe_group_wpb,
                                                   t.probe_group_warps, run[PB_LANES] ? 1 : 0, st);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;

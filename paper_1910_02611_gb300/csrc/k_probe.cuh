@@ -46,7 +46,8 @@ __host__ __device__ inline bool probe_short(uint64_t n, uint64_t total, int seq,
     return group <= 1 && total <= cut + PB_SHORT_MEAN * n;
 }
 
-// The instance that serves a batch (P: its warps per query).
+// The instance that serves a batch (P: its warps per query; wpb and
+// group_warps: of PB_GROUP's launch, whose blocks may be wider than the others').
 __host__ __device__ inline int probe_mode(const BatchView& b, int group, unsigned wpb, uint64_t group_warps, int lanes,
                                           unsigned& P) {
     P = 1;
@@ -238,7 +239,7 @@ __device__ __forceinline__ bool probe_group(const IndexView& ix, const HashParam
 
 template <int V, int G, int ETA, int MODE>
 __global__ void __launch_bounds__(QK_THREADS_MAX, RF * ETA * V <= 64 ? 2 : 1)
-    k_probe(IndexView ix, HashParams hp, BatchView b, QueryOut o, int batch, int order, int group,
+    k_probe(IndexView ix, HashParams hp, BatchView b, QueryOut o, int batch, int order, int group, int group_wpb,
             unsigned long long group_warps, int lanes, DevStatus* st) {
     const unsigned lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const unsigned grp = lane / G, slot = lane % G;
@@ -247,7 +248,7 @@ __global__ void __launch_bounds__(QK_THREADS_MAX, RF * ETA * V <= 64 ? 2 : 1)
     bv_resolve(b);
     if (query_batch_rejected(b, st)) return;
     unsigned P;
-    const int mode = probe_mode(b, group, blockDim.x >> 5, group_warps, lanes, P);
+    const int mode = probe_mode(b, group, (unsigned)group_wpb, group_warps, lanes, P);
     const bool listed = MODE == PB_WARP && mode == PB_LANES;  // the long queries that lane groups listed
     if (mode != MODE && !listed) return;
     if (b.n < PB_MANY && order == 2) order = 1;

@@ -12,7 +12,7 @@
 
 namespace rgb {
 
-using ProbeKernel = void (*)(IndexView, HashParams, BatchView, QueryOut, int, int, int, unsigned long long, int,
+using ProbeKernel = void (*)(IndexView, HashParams, BatchView, QueryOut, int, int, int, int, unsigned long long, int,
                              DevStatus*);
 
 ProbeKernel QK_CAT(probe_kernel_, QK_SUFFIX)(int V, int G, int mode) {

@@ -164,7 +164,8 @@ struct rambo {
     // and set kernels'
     struct Tuned {
         int wpb = 0, per_sm = 0, per_sm_g = 0;                    // query kernel
-        int probe_wpb = 0, probe_per_sm = 0, probe_per_sm_g = 0, probe_per_sm_l = 0;  // probe kernel
+        int probe_wpb = 0, probe_per_sm = 0, probe_per_sm_l = 0;  // probe kernel
+        int probe_wpb_g[2] = {}, probe_per_sm_g[2] = {};          // its grouped instance: the widest blocks, and as wide as the others'
         SetLaunch set{};
     } tuned;
     rambo_query_config_t tuned_cfg{};
@@ -616,9 +617,12 @@ void resolve_probe(rambo* h) {
         if (!ok || u.probe_per_sm_l < 1) u.set.qw = 0;
         u.probe_per_sm = std::min(u.probe_per_sm, most);
         u.probe_per_sm_l = std::min(u.probe_per_sm_l, most);
-        if (ok && group != 1 && u.probe_wpb > 1)
-            u.probe_per_sm_g = std::min(most, probe_max_blocks_per_sm(V, G, h->eta, PB_GROUP, u.probe_wpb,
-                                                                      probe_group_smem_bytes(h->R, h->S, u.probe_wpb)));
+        for (int i = 0; ok && group != 1 && i < 2; ++i) {
+            const int w = u.probe_wpb_g[i] = i || h->cfg.warps_per_block ? u.probe_wpb : 8;
+            if (w > 1)
+                u.probe_per_sm_g[i] = std::min(most, probe_max_blocks_per_sm(V, G, h->eta, PB_GROUP, w,
+                                                                             probe_group_smem_bytes(h->R, h->S, w)));
+        }
     }
     h->probe_known = true;
 }
@@ -688,10 +692,16 @@ int resolve_tuning(rambo* h, uint64_t n, int& use_bitmap, QueryTuning& t, bool p
         blocks = (uint64_t)u.probe_per_sm * h->num_sms;
         need = (n + t.probe_warps - 1) / t.probe_warps;
         t.probe_blocks = (int)(blocks < need ? blocks : need);
-        bg = (uint64_t)u.probe_per_sm_g * h->num_sms;
+        // as many warps a query as there can be: the widest blocks, unless a
+        // grid of them has no two warps for each query (rows of one word, whose
+        // other instances run best in blocks of four warps, 15000 k-mers of one
+        // query: 114 us by eight warps, 196 by four)
+        const int gi = t.group > 1 || 2 * n <= (uint64_t)u.probe_per_sm_g[0] * h->num_sms * u.probe_wpb_g[0] ? 0 : 1;
+        t.probe_group_wpb = u.probe_wpb_g[gi];
+        bg = (uint64_t)u.probe_per_sm_g[gi] * h->num_sms;
         if (bg > n) bg = n;
         t.probe_blocks_group = (int)bg;
-        t.probe_group_warps = bg * (uint64_t)t.probe_warps;
+        t.probe_group_warps = bg * (uint64_t)t.probe_group_wpb;
         // (a warp of the lane-group instance has 32 / G queries in flight)
         blocks = (uint64_t)u.probe_per_sm_l * h->num_sms;
         need = (n + (uint64_t)t.probe_warps * 32 / t.G - 1) / ((uint64_t)t.probe_warps * 32 / t.G);

@@ -371,6 +371,7 @@ struct QueryTuning {
     SetLaunch set;         // the set kernel's launch (qw = 0: this tuning keeps the set stage in the query kernel)
     int probe_warps, probe_batch;  // the probe kernel's counterparts
     int probe_blocks, probe_blocks_group, probe_blocks_lanes;
+    int probe_group_wpb;                   // warps of a block of its grouped instance
     unsigned long long probe_group_warps;
 };
 
