@@ -412,7 +412,7 @@ SetLaunch set_launch_shape(const IndexView& ix, int num_sms) {
         sl.smem = table * sl.qw;
     } else {
         const size_t one = (size_t)ix.R * ix.W * 32 * 4;  // a bit per cell for each of 32 queries
-        sl.qw = 4 * one <= QS_SMEM_TWO ? 4 : 2 * one <= QS_SMEM_TWO ? 2 : 4 * one <= QS_SMEM_MOST ? 4 : one <= QS_SMEM_MOST ? 1 : 0;
+        sl.qw = 4 * one <= QS_SMEM_TWO ? 4 : 2 * one <= QS_SMEM_TWO ? 2 : one <= QS_SMEM_MOST ? 1 : 0;
         sl.smem = one * sl.qw;
     }
     if (!sl.qw) return sl;
