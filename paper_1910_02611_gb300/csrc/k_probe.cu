@@ -42,10 +42,11 @@ cudaError_t launch_probe(const IndexView& ix, const HashParams& hp, const BatchV
     // are not worth the third one: they rarely have just eight k-mers).
     const int group = t.probe_blocks_group > 0 ? t.group : 1;
     bool run[3] = {true, t.probe_blocks_group > 0, !(b.desc && b.seq) && group <= 1 && b.n >= PB_MANY};
-    if (b.ends && qk_group_size(b.n, group, (unsigned)t.probe_group_wpb, t.probe_group_warps, 1) == 1) run[PB_GROUP] = false;
+    const unsigned wpb = (unsigned)t.probe_group_wpb;
+    if (b.ends && qk_group_size(b.n, group, wpb, t.probe_group_warps, 1) == 1) run[PB_GROUP] = false;
     if (!b.desc && !b.ends) {
         unsigned P;
-        const int mode = probe_mode(b, group, (unsigned)t.probe_group_wpb, t.probe_group_warps, 1, P);
+        const int mode = probe_mode(b, group, wpb, t.probe_group_warps, 1, P);
         for (int m = 0; m < 3; ++m) run[m] = m == mode;
         // with lane groups, also for queries longer than they take, if there can be one
         const uint64_t least = b.seq ? b.k : 1;

@@ -57,8 +57,11 @@ __host__ __device__ inline int probe_mode(const BatchView& b, int group, unsigne
 }
 
 // Row reads use the default cache operator alone (read-only path, no L1
-// allocation, 64-byte L2 fetch; row_load 7): the switch over the eight of them
-// at each of a step's R * eta reads made the kernel spill.
+// allocation, 64-byte L2 fetch; row_load 7): a switch over the eight of them
+// at each of a step's R * eta reads made the kernel spill.  What spills all
+// the same, at 128 registers: instances of V = 4 and eta <= 2 (8 to 64 bytes;
+// 44 in <4, 1, 2, PB_WARP>, rows of 16 bytes) and the lane groups of eta > 2
+// (40 to 120).
 template <int V>
 __device__ __forceinline__ void probe_load(const uint32_t* p, uint32_t (&v)[V]) {
     if constexpr (V == 1)

@@ -1,9 +1,10 @@
 // k_query_set.cu -- the set stage (Algorithm 2's union per table and
-// intersection across tables) of the queries whose masks leave many candidate
-// sets, 32 * QW of them at a time.
+// intersection across tables) of batches on the probe path, 32 * QW queries at
+// a time.
 //
-// The query kernel hands such a query over as its R per-table cell masks.  A
-// block takes 32 * QW queries and transposes their masks in shared memory, so
+// The probe kernels (k_probe.cuh, k_query_wide.cu) hand over every query whose
+// R per-table cell masks all keep a hit cell, as those masks.  A block takes
+// 32 * QW of them and transposes their masks in shared memory, so
 // that T[r][cell] holds one bit per query: bit q = cell is hit in table r for
 // query q.  A set i then needs one shared-memory read per table for all of
 // them,

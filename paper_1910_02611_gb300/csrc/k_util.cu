@@ -747,6 +747,7 @@ __device__ __forceinline__ uint32_t ga_parts(uint32_t bits_words, uint64_t n, ui
     return parts > base ? parts : base;
 }
 
+// (six blocks an SM: 40 registers, of which a cut answer's path spills 68 bytes)
 __global__ void __launch_bounds__(GA_THREADS, 6) k_gather(QueryOut o, const uint64_t* __restrict__ id_offsets, uint64_t n,
                                                         uint32_t* __restrict__ ids, DevStatus* st,
                                                         const uint64_t* __restrict__ n_dev, uint64_t ids_cap) {

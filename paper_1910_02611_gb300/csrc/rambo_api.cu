@@ -165,7 +165,8 @@ struct rambo {
     struct Tuned {
         int wpb = 0, per_sm = 0, per_sm_g = 0;                    // query kernel
         int probe_wpb = 0, probe_per_sm = 0, probe_per_sm_l = 0;  // probe kernel
-        int probe_wpb_g[2] = {}, probe_per_sm_g[2] = {};          // its grouped instance: the widest blocks, and as wide as the others'
+        // its grouped instance: the widest blocks, and blocks as wide as the others'
+        int probe_wpb_g[2] = {}, probe_per_sm_g[2] = {};
         SetLaunch set{};
     } tuned;
     rambo_query_config_t tuned_cfg{};

@@ -292,10 +292,12 @@ int rambo_plan_create(rambo_t* h, int kind, uint64_t max_queries, uint64_t max_i
     // arena above (or 256 MiB) and a quarter of the memory that is free now
     // that the plan has all it needs without them; they then take the arena's
     // place.
-    const uint64_t words = max_queries * set_pitch(ix.K), masks = max_queries * ix.R * ix.S, extra = words + masks + 2 * max_queries;
+    const uint64_t words = max_queries * set_pitch(ix.K), masks = max_queries * ix.R * ix.S;
+    const uint64_t extra = words + masks + 2 * max_queries;
     const uint64_t most = p->stage_words * 4 > (64ull << 20) ? p->stage_words * 4 : 64ull << 20;
     size_t free_b = 0, total_b = 0;
-    if (t.set.qw && extra <= most && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && extra <= (uint64_t)free_b / 16) {
+    if (t.set.qw && extra <= most && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess &&
+        extra <= (uint64_t)free_b / 16) {
         uint32_t* stage = nullptr;
         p->probe = cudaMalloc(&stage, words * 4) == cudaSuccess && cudaMalloc(&p->dmask, masks * 4) == cudaSuccess &&
                    cudaMalloc(&p->dq, max_queries * 8) == cudaSuccess;
