@@ -16,7 +16,8 @@
 //
 // What bounds it: the shared-memory pipe.  32 IDs x 128 queries cost R 16-byte
 // reads a lane at random cells (8.6 wavefronts each, measured) and 20 shuffles;
-// ncu shows 64% of the pipe's wavefronts and 3 blocks an SM.  Measured, set
+// on 2e4 document queries ncu shows 75% of the L1 and shared data pipe's
+// wavefronts, 55% by shared memory alone, and 3 blocks an SM.  Measured, set
 // stage with the probes before it, against one query per warp in the query
 // kernel: 1e5 conjunctive queries over 1e5 documents (R = 8, B = 320) 11.7 ms
 // -> 0.26 (probes) + 0.89; 1e4 over 5e5 documents (R = 6, B = 1000; no

@@ -763,10 +763,13 @@ __global__ void __launch_bounds__(GA_THREADS, 6) k_gather(QueryOut o, const uint
     const uint64_t units = n * parts;
     // answers that are cut into many parts are taken a part at a time, so that
     // a long one's parts go to several warps, and whole ones no more at a time
-    // than leaves every warp some; the first take needs no ticket
+    // than gives every warp some.  The first take needs no ticket, and none is
+    // drawn where the first takes are all there is (1e4 tickets from one
+    // counter: 5 us)
     const unsigned take = units >= warps * GA_TAKE ? (parts == 1 ? GA_TAKE : parts < 8 ? GA_TAKE / 2 : 1)
-                          : parts == 1             ? max(1u, (unsigned)(units / warps))
+                          : parts == 1             ? (unsigned)((units + warps - 1) / warps)
                                                    : 1;
+    const bool once = units <= warps * take;
     for (unsigned long long u0 = ((uint64_t)blockIdx.x * GA_WARPS + (threadIdx.x >> 5)) * take; u0 < units;) {
         // a lane looks up each unit of the ticket, then the warp takes them one by one
         uint32_t c_of = 0, part_of = 0;
@@ -803,6 +806,7 @@ __global__ void __launch_bounds__(GA_THREADS, 6) k_gather(QueryOut o, const uint
             }
             ga_expand(src, w_lo, w_hi, dst, run, lane);
         }
+        if (once) break;
         if (lane == 0) u0 = warps * take + atomicAdd(&st->gather_ticket, (unsigned long long)take);
         u0 = __shfl_sync(FULL, u0, 0);
     }
