@@ -12,7 +12,6 @@
 // streams against the same (read-only) index.
 #include <cstring>
 #include <new>
-#include <utility>
 
 #include "k_query.cuh"
 #include "rambo_impl.cuh"
@@ -266,14 +265,41 @@ int rambo_plan_create(rambo_t* h, int kind, uint64_t max_queries, uint64_t max_i
         return code;
     };
     if (cudaSetDevice(p->device) != cudaSuccess) return fail(RAMBO_ECUDA);
+    // On the probe path every answer is staged as a bitmap of set_pitch(K)
+    // words and handed over as R * S words of masks.  It is taken when an
+    // arena and masks for max_queries of them are no more than four times the
+    // arena above (or 256 MiB) and a quarter of the memory that stays free
+    // when the plan has all that it needs without them.
+    const uint64_t packed = kind == 1 ? max_items / 32 + 2 : 0, scan = scan_tmp_words(max_queries);
+    const uint64_t need = max_items * p->elem + 16 + packed * (p->skipn ? 12 : 8) + max_queries * 28 + 16 + scan * 8 +
+                          (p->stage_words + max_ids) * 4 + sizeof(PlanHead);
+    const uint64_t words = max_queries * set_pitch(ix.K), masks = max_queries * ix.R * ix.S;
+    const uint64_t extra = words + masks + 2 * max_queries;
+    const uint64_t most = p->stage_words * 4 > (64ull << 20) ? p->stage_words * 4 : 64ull << 20;
+    size_t free_b = 0, total_b = 0;
+    if (t.set.qw && extra <= most && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && free_b > need &&
+        extra <= ((uint64_t)free_b - need) / 16) {
+        p->probe = cudaMalloc(&p->stage, words * 4) == cudaSuccess && cudaMalloc(&p->dmask, masks * 4) == cudaSuccess &&
+                   cudaMalloc(&p->dq, max_queries * 8) == cudaSuccess;
+        if (p->probe) {
+            p->stage_words = words;
+        } else {
+            cudaGetLastError();
+            for (uint32_t** d : {&p->stage, &p->dmask, &p->dq}) {
+                if (*d) cudaFree(*d);
+                *d = nullptr;
+            }
+        }
+    }
     bool ok = cudaMalloc(&p->d_data, max_items * p->elem + 16) == cudaSuccess &&
               cudaMalloc(&p->d_off, (max_queries + 1) * 8) == cudaSuccess &&
-              (kind == 0 || cudaMalloc(&p->d_packed, (max_items / 32 + 2) * 8) == cudaSuccess) &&
-              (!p->skipn || cudaMalloc(&p->d_nmask, (max_items / 32 + 2) * 4) == cudaSuccess) &&
+              (kind == 0 || cudaMalloc(&p->d_packed, packed * 8) == cudaSuccess) &&
+              (!p->skipn || cudaMalloc(&p->d_nmask, packed * 4) == cudaSuccess) &&
               cudaMalloc(&p->qcount, max_queries * 4) == cudaSuccess &&
               cudaMalloc(&p->qstart, max_queries * 8) == cudaSuccess &&
-              cudaMalloc(&p->scan_tmp, scan_tmp_words(max_queries) * 8) == cudaSuccess &&
-              cudaMalloc(&p->stage, p->stage_words * 4) == cudaSuccess && cudaMalloc(&p->ids, max_ids * 4) == cudaSuccess &&
+              cudaMalloc(&p->scan_tmp, scan * 8) == cudaSuccess &&
+              (p->probe || cudaMalloc(&p->stage, p->stage_words * 4) == cudaSuccess) &&
+              cudaMalloc(&p->ids, max_ids * 4) == cudaSuccess &&
               cudaMalloc(&p->id_off, (max_queries + 1) * 8) == cudaSuccess &&
               cudaMalloc(&p->d_head, sizeof(PlanHead)) == cudaSuccess &&
               cudaMallocHost(&p->h_data, max_items * p->elem + 16) == cudaSuccess &&
@@ -285,33 +311,6 @@ int rambo_plan_create(rambo_t* h, int kind, uint64_t max_queries, uint64_t max_i
     if (!ok) {
         cudaGetLastError();
         return fail(RAMBO_ENOMEM);
-    }
-    // On the probe path every answer is staged as a bitmap of set_pitch(K)
-    // words and handed over as R * S words of masks.  It is taken when an
-    // arena and masks for max_queries of them are no more than four times the
-    // arena above (or 256 MiB) and a quarter of the memory that is free now
-    // that the plan has all it needs without them; they then take the arena's
-    // place.
-    const uint64_t words = max_queries * set_pitch(ix.K), masks = max_queries * ix.R * ix.S;
-    const uint64_t extra = words + masks + 2 * max_queries;
-    const uint64_t most = p->stage_words * 4 > (64ull << 20) ? p->stage_words * 4 : 64ull << 20;
-    size_t free_b = 0, total_b = 0;
-    if (t.set.qw && extra <= most && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess &&
-        extra <= (uint64_t)free_b / 16) {
-        uint32_t* stage = nullptr;
-        p->probe = cudaMalloc(&stage, words * 4) == cudaSuccess && cudaMalloc(&p->dmask, masks * 4) == cudaSuccess &&
-                   cudaMalloc(&p->dq, max_queries * 8) == cudaSuccess;
-        if (p->probe) {
-            std::swap(stage, p->stage);
-            p->stage_words = words;
-        } else {
-            cudaGetLastError();
-            for (uint32_t** d : {&p->dmask, &p->dq}) {
-                if (*d) cudaFree(*d);
-                *d = nullptr;
-            }
-        }
-        if (stage) cudaFree(stage);
     }
     p->st = &p->d_head->st;
     p->d_desc = p->d_head->desc;
