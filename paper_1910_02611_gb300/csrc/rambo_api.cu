@@ -693,11 +693,15 @@ int resolve_tuning(rambo* h, uint64_t n, int& use_bitmap, QueryTuning& t, bool p
         blocks = (uint64_t)u.probe_per_sm * h->num_sms;
         need = (n + t.probe_warps - 1) / t.probe_warps;
         t.probe_blocks = (int)(blocks < need ? blocks : need);
-        // as many warps a query as there can be: the widest blocks, unless a
-        // grid of them has no two warps for each query (rows of one word, whose
-        // other instances run best in blocks of four warps, 15000 k-mers of one
-        // query: 114 us by eight warps, 196 by four)
-        const int gi = t.group > 1 || 2 * n <= (uint64_t)u.probe_per_sm_g[0] * h->num_sms * u.probe_wpb_g[0] ? 0 : 1;
+        // the widest blocks where they give a query more warps (rows of one
+        // word, whose other instances run best in blocks of four warps, 15000
+        // k-mers of one query: 114 us by eight warps, 196 by four); by as many
+        // warps in narrower ones 400 queries of 970 took 37 us against 39
+        unsigned P[2];
+        for (int i = 0; i < 2; ++i)
+            P[i] = query_group_size(n, t.group, (unsigned)u.probe_wpb_g[i],
+                                    std::min<uint64_t>((uint64_t)u.probe_per_sm_g[i] * h->num_sms, n) * u.probe_wpb_g[i], 1);
+        const int gi = P[0] > P[1] ? 0 : 1;
         t.probe_group_wpb = u.probe_wpb_g[gi];
         bg = (uint64_t)u.probe_per_sm_g[gi] * h->num_sms;
         if (bg > n) bg = n;
