@@ -450,7 +450,7 @@ int rambo_last_query_stats(const rambo_t *h, rambo_query_stats_t *out);
  *   blocks_per_sm (0 = as many as fit),
  *   set_stage: 0 = auto (batches of more than the smallest size: probe and set
  *              kernels, when row_load and answer_staging are at their
- *              defaults too and memory holds a bitmap a query),
+ *              defaults too and memory holds bitmap and masks of each),
  *              1 = dense scan of the partition table,
  *              2 = sparse enumeration of the hit cells' members,
  *              3 = union of the hit cells' member bitmaps (complemented for

@@ -88,8 +88,9 @@ __device__ __forceinline__ void bk_records(const IndexView& ix, const HashParams
 // a record costs two shared atomics, one store and one load.  A bucket that would overflow sets *overflow
 // instead (the caller then files the chunk again).
 //
-// What bounds it: instruction issue (70% of the slots), then the shared-memory
-// pipe (46%: the atomics and the scattered stores).  Measured on 2e9 k-mers
+// What bounds it: instruction issue (64% of the slots with 64 windows), then the
+// shared-memory pipe (55%: the atomics and the scattered stores; 76% with 8
+// windows, where a warp's lanes meet on the same counters).  Measured on 2e9 k-mers
 // with R * eta = 12 (2.4e10 records, 128 windows): 181 -> 60.6 ms.  Staging
 // every record with its window, two blocks of 256 threads an SM and a search
 // for the item every step made up the 181; one multiplication for the window
